@@ -284,10 +284,9 @@ int deam_init(const deam_geometry* geom, const deam_spectra* spectra, const deam
     ctx->delta = o.penalty_lambda > 0.0 ? o.penalty_delta : 1.0;
     ctx->threshold = o.metal_threshold > 0.0 ? o.metal_threshold
                                              : 0.5 * std::min(g.dx, std::min(g.dy, g.nz > 1 ? g.dz : g.dx));
-    ctx->slab = deam::context_slab(deam::pick_slab(g.nz, g.n_rows, g.dz, g.row_pitch, g.sid, g.sdd));
-    ctx->n_slabs = (g.nz + ctx->slab - 1) / ctx->slab;
     int sms = 152;
     cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, ctx->device);
+    ctx->bwd = deam::bwd_plan(g.nx, g.ny, g.nz, deam::pick_slab(g.nz, g.n_rows, g.dz, g.row_pitch, g.sid, g.sdd), sms);
     const long long ntiles = (long long)((g.n_channels + deam::kTileK - 1) / deam::kTileK) *
                              ((g.n_rows + deam::kTileR - 1) / deam::kTileR) *
                              ((g.n_views + deam::kTileV - 1) / deam::kTileV);
@@ -315,7 +314,7 @@ int deam_init(const deam_geometry* geom, const deam_spectra* spectra, const deam
         rw[r] = make_float2((float)(w / g.dz), (float)sqrt(1.0 + (w / g.sdd) * (w / g.sdd)));
     }
     // per (slab, column tile) in the backprojector's block order
-    const std::vector<int2> sv = deam::tile_view_ranges(g, ctx->slab, deam::kTileX, deam::kTileY);
+    const std::vector<int2> sv = deam::tile_view_ranges(g, ctx->bwd.slab, deam::bwd_tile_x(ctx->bwd.vs), deam::bwd_tile_y(ctx->bwd.vs));
 
     Geo& G = ctx->G;
     G.nx = g.nx; G.ny = g.ny; G.nz = g.nz; G.V = g.n_views; G.R = g.n_rows; G.K = g.n_channels;
@@ -327,6 +326,7 @@ int deam_init(const deam_geometry* geom, const deam_spectra* spectra, const deam
     G.chan_c0 = (float)((g.n_channels - 1) / 2.0 - g.channel_offset);
     G.inv_dgamma = (float)(1.0 / g.channel_pitch);
     G.vox_reach_mm = (float)(std::max(g.dx, g.dy) * 1.001);
+    G.inv_sdd = (float)(1.0 / g.sdd);
 
     // ---- spectral tables ----
     Spec& S = ctx->S;
@@ -555,7 +555,7 @@ int deam_backproject(deam_ctx* ctx, const float* y, float* img, void* stream) {
     B.rays2 = (const float2*)y;
     B.img = (float2*)img;
     B.slab_views = ctx->slab_views;
-    CK(deam::launch_backward(deam::BWD_ADJOINT, ctx->slab, ctx->G, B, (cudaStream_t)stream));
+    CK(deam::launch_backward(deam::BWD_ADJOINT, ctx->bwd, ctx->G, B, (cudaStream_t)stream));
     return deam::finish_call(ctx, (cudaStream_t)stream);
 }
 
@@ -663,7 +663,7 @@ int deam_iterate(deam_ctx* ctx, float* c, int n_iter, double* hist, void* stream
         if (e) CK(cudaEventRecord(e[3], s));
         {
             NvtxRange r("deam.backproject");  // gather backprojection + c-step
-            CK(deam::launch_backward(deam::BWD_UPDATE, ctx->slab, ctx->G, B, s));
+            CK(deam::launch_backward(deam::BWD_UPDATE, ctx->bwd, ctx->G, B, s));
             if (B.sums) CK(deam::launch_reg_update(ctx->G, B, s));
         }
         if (e) CK(cudaEventRecord(e[4], s));
@@ -710,7 +710,7 @@ int deam_backprojected_sums(deam_ctx* ctx, const float* c, float* sums, double* 
     B.payload = ctx->payload;
     B.slab_views = ctx->slab_views;
     B.sums = (float4*)sums;  // the c-step's backprojection, stopped before the update
-    CK(deam::launch_backward(deam::BWD_UPDATE, ctx->slab, ctx->G, B, s));
+    CK(deam::launch_backward(deam::BWD_UPDATE, ctx->bwd, ctx->G, B, s));
     rc = deam::finish_call(ctx, s);
     if (rc != DEAM_OK) return rc;
     if (Z) *Z = ctx->Z;
@@ -738,7 +738,7 @@ int deam_gradient(deam_ctx* ctx, const float* c, float* grad, double* F, void* s
     B.payload = ctx->payload;
     B.img = (float2*)grad;
     B.slab_views = ctx->slab_views;
-    CK(deam::launch_backward(deam::BWD_GRADIENT, ctx->slab, ctx->G, B, s));
+    CK(deam::launch_backward(deam::BWD_GRADIENT, ctx->bwd, ctx->G, B, s));
     rc = deam::finish_call(ctx, s);
     if (rc != DEAM_OK) return rc;
     if (F) {

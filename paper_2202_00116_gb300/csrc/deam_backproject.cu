@@ -10,365 +10,377 @@
 
 namespace deam {
 
-// Voxel-driven gather backprojection.  A block owns a kTileX x kTileY tile of
-// (ix, iy) columns and a z-slab of SLAB voxels; each thread owns one column and
-// keeps its SLAB accumulators in shared memory (layout [slot][thread], so a
-// warp's accesses to one slot are conflict-free).  For every view that can reach
-// the slab, the thread takes the channels whose rays can touch its column (fan
-// angle of the column centre +- the footprint), evaluates each such ray's sample
-// at its plane exactly as the forward kernel does (same in-plane table, same
-// explicitly rounded t(p), omega_r and fz), and for every row whose sample falls
-// in the slab adds h(x, y) * payload(y) to the two voxels the sample
-// interpolates.  The kernel lives on the L1/shared-memory data path (the
-// accumulator read-modify-writes and the payload gathers) and on the latency
-// of its gathers, so the row loop reads nothing but the payload: omega_r is
-// computed, and the payload already carries h's row length factor.  Views are taken in pairs: the samples of one row from
-// two consecutive views lie within a few hundredths of a slice of each other,
-// so they almost always fall in the same slot pair, and one read-modify-write
-// of each slot adds both (half the accumulator traffic).  With 8-slice slabs
-// (several rows per slice) consecutive rows share a slot pair instead, which
-// is kept in registers.
-constexpr int kBwdThreads = kTileX * kTileY;
+// Voxel-driven gather backprojection.  A thread owns one (ix, iy) column and the
+// SLAB slices of one z-slab, whose sums it keeps in shared memory ([slot][thread]:
+// conflict-free).  A warp owns an 8 x 4 patch of columns and takes the views that
+// can reach its slab two at a time: the channels whose rays tap a column come
+// from the fan angles of the patch's corners, and then a row of the detector is
+// one turn of the loop, which adds the samples of all the rays of both views
+// (2.6 rays per view and column at 512^2 x 816 channels).  These lie within a few
+// hundredths of a slice of each other, so nearly always all between the same two
+// slices, and one read and write of these two serves them all.  Sample positions
+// are the forward kernel's, bit for bit (same in-plane table, same explicitly
+// rounded t(p), omega_r and fz).
+//
+// What bounds it: issue (0.6 per cycle and scheduler) and the latency of the
+// payload gathers with the 20 warps per SM that 96 registers allow, the L1 data
+// path being 60-70 % busy.  One ray at a time (two views abreast) cost twice the
+// shared-memory traffic, half the loads in flight and 70 instead of 31
+// instructions per (column, ray, row): 37.4 -> 22.9 ms on one rotation of the
+// 512^2 x 64 scan, 20.5 -> 8.6 ms on one of the 256^2 x 32 scan.  Measured and
+// slower: sums in registers with the slices unrolled (37.5 ms on the first),
+// four views per turn (29-50 ms), first moments of the rays' heights instead of
+// each ray's own weights (faster by 5 % but no longer the forward's weights).
+constexpr int kBwdThreads = 128;
+// Rays of a view that one turn of the row loop takes (more rays: more turns).
+// Four at 5 blocks of 128 threads per SM; three at 6 blocks are as fast at 2.6
+// rays per view and 8 % slower at 3.5 (384^2 x 48 on 816 channels).
+constexpr int kRaysPerView = 4;
 
-__device__ __forceinline__ float channel_coord(const Geo& G, float4 vw, float x, float y, float* dist) {
-    const float px = (x - vw.x) * G.dx, py = (y - vw.y) * G.dy;
-    const float dot = -(px * vw.z + py * vw.w);
-    const float crs = px * vw.w - py * vw.z;
-    if (dist) *dist = sqrtf(dot * dot + crs * crs);
-    return fmaf(atan2f(crs, dot), G.inv_dgamma, G.chan_c0);
+typedef unsigned long long pair32;  // two FP32 values in a register pair
+
+__device__ __forceinline__ pair32 pack2(float x, float y) {
+    pair32 r;
+    asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(x), "f"(y));
+    return r;
+}
+__device__ __forceinline__ float2 unpack2(pair32 v) {
+    float2 r;
+    asm("mov.b64 {%0, %1}, %2;" : "=f"(r.x), "=f"(r.y) : "l"(v));
+    return r;
+}
+// a b + c on both halves, each rounded as fmaf rounds it
+__device__ __forceinline__ pair32 fma2(pair32 a, pair32 b, pair32 c) {
+    pair32 d;
+    asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(d) : "l"(a), "l"(b), "l"(c));
+    return d;
 }
 
-template <bool FOUR, int SLAB, int NT>
-__device__ __forceinline__ void pend_flush(float4* acc, int s, int tid, float4 x) {
-    if (s >= 0 && s < SLAB) {
-        float4& a = acc[s * NT + tid];
-        a.x += x.x;
-        a.y += x.y;
-        if (FOUR) {
-            a.z += x.z;
-            a.w += x.w;
-        }
-    }
+__device__ __forceinline__ pair32 add2(pair32 a, pair32 b) {
+    pair32 d;
+    asm("add.rn.f32x2 %0, %1, %2;" : "=l"(d) : "l"(a), "l"(b));
+    return d;
 }
+__device__ __forceinline__ pair32 dup2(float x) { return pack2(x, x); }
 
-
-// One ray's visit of a column: what the row loop needs.
-struct ColRay {
-    long long pb;  // ray-data index of row 0: (v R) K + k
-    float sz;      // sigma_z of the view
-    float tp;      // ray parameter at the column's plane
-    float Lq;      // Joseph length x in-plane bilinear weight (0: the ray misses the column)
-    int r0, r1;    // rows whose sample can land in the slab (r0 > r1: none)
+// A ray's data, or the sums of a voxel: (b~_1, b~_2) and, for the c-step, also
+// (delta_1, delta_2).  The gradient carries the second pair alone, the plain
+// adjoint its two components.
+template <bool FOUR>
+struct Sums {
+    pair32 a, b;
+};
+template <>
+struct Sums<false> {
+    pair32 a;
 };
 
-// Channel window [k0, k1] of view v for the column at (fix, fiy) (k0 > k1:
-// none), and the view's sigma_z.
-__device__ __forceinline__ void view_window(const Geo& G, int v, float fix, float fiy, int& k0, int& k1, float& sz) {
-    const float4 vw = __ldg(&G.view4[v]);
-    sz = __ldg(&G.view_z[v]);
-    float dist;
-    const float uc = channel_coord(G, vw, fix, fiy, &dist);
-    // a ray can tap the column only if it passes within one voxel edge of its
-    // centre: |gamma - gamma_c| < asin(edge / dist) < reach / (dist - reach);
-    // 0.05 channel of margin covers the FP32 channel coordinate
-    const float hw = __fdividef(G.vox_reach_mm, fmaxf(dist - G.vox_reach_mm, 1.f)) * G.inv_dgamma + 0.05f;
-    k0 = max(0, (int)ceilf(fmaxf(uc - hw, -1.f)));
-    k1 = min(G.K - 1, (int)floorf(fminf(uc + hw, (float)G.K)));
-    if (!DEAM_IN_BOUNDS(G, k0 > k1 || (k0 >= 0 && (long long)v * G.K + k1 < (long long)G.V * G.K), SITE_BWD_TABLE,
-                        (long long)v * G.K + k1))
-        k1 = k0 - 1;
-}
-
-__device__ __forceinline__ ColRay no_ray() {
-    ColRay c;
-    c.pb = 0;
-    c.sz = 0.f;
-    c.tp = 0.f;
-    c.Lq = 0.f;
-    c.r0 = 0;
-    c.r1 = -1;
-    return c;
-}
-
-// Ray (v, k) at column (ix, iy), from its in-plane table entry (a4, aL): the
-// sample at the column's plane exactly as the forward kernel evaluates it;
-// Lq = 0 when the ray does not touch the column.
-__device__ __forceinline__ ColRay col_ray(const Geo& G, int v, int k, float4 a4, float aL, int ix, int iy, float sz,
-                                          float zlo, float zhi) {
-    ColRay c;
-    c.pb = (long long)v * G.R * G.K + k;
-    c.sz = sz;
-    c.Lq = 0.f;
-    c.tp = 0.f;
-    c.r0 = 0;
-    c.r1 = -1;
-    const InPlane ip = inplane_at(a4, aL);
-    const int p = ip.axis ? iy : ix;
-    const int q = ip.axis ? ix : iy;
-    const float pf = (float)p;
-    const float fq = __fmaf_rn(pf, ip.bq, ip.aq);
-    const float jq = floorf(fq);
-    const float aq = fq - jq;
-    float wq = 0.f;
-    if (jq == (float)q) wq = 1.f - aq;
-    else if (jq == (float)(q - 1)) wq = aq;
-    c.tp = ray_t(ip, pf);
-    if (wq == 0.f) return c;
-    int r0 = 0, r1 = G.R - 1;
-    if (G.R > 1) {
-        const float slope = c.tp * G.domega;
-        if (fabsf(slope) > 1e-20f) {
-            const float inv = __fdividef(1.f, slope);
-            const float base = fmaf(c.tp, G.omega0, sz);
-            const float ra = (zlo - base) * inv, rb = (zhi - base) * inv;
-            const float lo = fminf(fmaxf(fminf(ra, rb), -4.f), (float)G.R + 4.f);
-            const float hi = fminf(fmaxf(fmaxf(ra, rb), -4.f), (float)G.R + 4.f);
-            r0 = max(0, (int)floorf(lo - 0.02f));
-            r1 = min(G.R - 1, (int)ceilf(hi + 0.02f));
-        }
-    }
-    if (!DEAM_IN_BOUNDS(G, c.pb + (long long)(G.R - 1) * G.K < (long long)G.V * G.R * G.K, SITE_BWD_RAY,
-                        c.pb + (long long)(G.R - 1) * G.K))
-        return c;
-    c.Lq = ip.Lxy * wq;
-    c.r0 = r0;
-    c.r1 = r1;
-    return c;
-}
-
 template <int MODE>
-__device__ __forceinline__ float4 ray_payload(const BwdArgs& A, long long i) {
-    if (MODE == BWD_ADJOINT) {
-        const float2 t = __ldg(&A.rays2[i]);
-        return make_float4(t.x, t.y, 0.f, 0.f);
-    }
-    float4 P = __ldg(&A.payload[i]);
-    if (MODE == BWD_GRADIENT) P = make_float4(P.z, P.w, 0.f, 0.f);
+__device__ __forceinline__ Sums<MODE == BWD_UPDATE> ray_data(const BwdArgs& A, long long i) {
+    Sums<MODE == BWD_UPDATE> P;
+    if constexpr (MODE == BWD_UPDATE)
+        asm("ld.global.nc.v2.u64 {%0, %1}, [%2];" : "=l"(P.a), "=l"(P.b) : "l"(A.payload + i));
+    else if constexpr (MODE == BWD_GRADIENT)
+        asm("ld.global.nc.u64 %0, [%1 + 8];" : "=l"(P.a) : "l"(A.payload + i));
+    else
+        asm("ld.global.nc.u64 %0, [%1];" : "=l"(P.a) : "l"(A.rays2 + i));
     return P;
 }
 
-template <bool FOUR, int SLAB, int NT>
-__device__ __forceinline__ void slot_add(float4* acc, int s, int tid, float w, const float4& P) {
-    if (s >= 0 && s < SLAB) {
-        float4& a = acc[s * NT + tid];
-        a.x = fmaf(w, P.x, a.x);
-        a.y = fmaf(w, P.y, a.y);
-        if (FOUR) {
-            a.z = fmaf(w, P.z, a.z);
-            a.w = fmaf(w, P.w, a.w);
+// s + w P
+template <bool FOUR>
+__device__ __forceinline__ void add_scaled(Sums<FOUR>& s, pair32 w, const Sums<FOUR>& P) {
+    s.a = fma2(w, P.a, s.a);
+    if constexpr (FOUR) s.b = fma2(w, P.b, s.b);
+}
+template <bool FOUR>
+__device__ __forceinline__ void add_to(Sums<FOUR>& s, const Sums<FOUR>& P) {
+    s.a = add2(s.a, P.a);
+    if constexpr (FOUR) s.b = add2(s.b, P.b);
+}
+
+// Fan angle of a direction (dot along the central ray, crs across it).  Within
+// 31 degrees of the central ray (every fan of this scanner family) a degree-9
+// odd polynomial, the Chebyshev interpolant of atan(x) / x in x^2 on [0, 0.36]
+// (3e-7 rad); it only places the channel window, whose margin is larger by far.
+__device__ __forceinline__ float fan_angle(float crs, float dot) {
+    if (fabsf(crs) > 0.6f * dot) return atan2f(crs, dot);
+    const float r = __fdividef(crs, dot), x = r * r;
+    float s = 0.0578066558f;
+    s = fmaf(s, x, -0.128525928f);
+    s = fmaf(s, x, 0.198297724f);
+    s = fmaf(s, x, -0.333260238f);
+    s = fmaf(s, x, 0.999999464f);
+    return s * r;
+}
+
+// What a view asks of the 8 x 4 columns of a warp, seen from one of their corner
+// columns: the corner's channel coordinate u, the half width hw of a column's
+// channel window around its own coordinate, and the rows [lo, hi] (real numbers)
+// that can reach the slab.
+struct CornerWindow {
+    float u, hw, lo, hi;
+};
+
+__device__ __forceinline__ CornerWindow corner_window(const Geo& G, int v, float fix, float fiy, float zlo, float zhi) {
+    CornerWindow W;
+    const float4 vw = __ldg(&G.view4[v]);
+    const float sz = __ldg(&G.view_z[v]);
+    const float px = (fix - vw.x) * G.dx, py = (fiy - vw.y) * G.dy;
+    const float dot = -fmaf(px, vw.z, py * vw.w);
+    const float crs = fmaf(px, vw.w, -py * vw.z);
+    const float d2 = fmaf(px, px, py * py);
+    const float inv = rsqrtf(d2);
+    const float dist = d2 * inv;
+    const float rest = __fdividef(1.f, fmaxf(dist - G.vox_reach_mm, 1e-3f * dist));
+    const float rho = G.vox_reach_mm * rest;  // a voxel edge as an angle, a little over
+    // A ray taps a column if at the column's plane it passes within one voxel
+    // edge e of its centre, across the dominant axis: e |cos| of perpendicular
+    // distance, an angle below e |cos| / (dist - e).  Taking the larger of the
+    // two axes covers rays of either dominance.  What varies over the patch is
+    // covered by the corners up to second order in its angle (64 rho^2), and so is
+    // the error of interpolating u between them ((7^2 + 3^2) / 8 rho^2 as |u''| is
+    // at most 1 / (dist^2 dgamma)); 0.05 channel of margin covers the rounding.
+    // (The bound e / (dist - e), without the cosine, lets through up to 40 % more
+    // channels.)
+    const float edge = fmaxf(fabsf(px) * G.dy, fabsf(py) * G.dx) * inv * 1.001f;
+    const float bend = rho * rho;
+    W.hw = fmaf(fmaf(edge * rest, fmaf(64.f, bend, 1.f), 8.f * bend), G.inv_dgamma, 0.05f);
+    W.u = fmaf(fan_angle(crs, dot), G.inv_dgamma, G.chan_c0);
+    W.lo = 0.f;
+    W.hi = (float)(G.R - 1);
+    const float t = dist * G.inv_sdd, slope = t * G.domega;
+    if (G.R > 1 && slope > 1e-20f) {
+        // fz(r) = sigma_z + t (omega0 + r domega) with t = dist / sdd for a ray
+        // through the column's centre; the rays that tap it pass within one voxel
+        // edge, which moves t by at most rho of itself and the row of a height z by
+        // the same share of (z - sigma_z) / (t domega)
+        const float is = __fdividef(1.f, slope);
+        const float off = G.omega0 * t * is;
+        const float share = rho * fmaf(16.f, rho, 1.f);
+        const float ulo = (zlo - sz) * is, uhi = (zhi - sz) * is;
+        W.lo = ulo - off - fmaf(fabsf(ulo), share, 0.02f);
+        W.hi = uhi - off + fmaf(fabsf(uhi), share, 0.02f);
+    }
+    if (rho > 0.1f) {  // voxels too large for these bounds: every channel and row
+        W.u = 0.f;
+        W.hw = 1e9f;
+        W.lo = 0.f;
+        W.hi = (float)(G.R - 1);
+    }
+    return W;
+}
+
+// G neighbouring rays (v, k .. k + G - 1) at a column: Joseph length x in-plane
+// weight (0: the ray does not tap the column) and ray parameter.
+template <int G_>
+struct Rays {
+    float c[G_], t[G_];
+};
+
+template <int G_>
+__device__ __forceinline__ void load_rays(const Geo& G, Rays<G_>& y, int v, int k, int k1, float fix, float fiy,
+                                          float& tmin, float& tmax) {
+    const long long vk = (long long)v * G.K + k;
+#pragma unroll
+    for (int g = 0; g < G_; ++g) {
+        y.c[g] = y.t[g] = 0.f;
+        if (k + g <= k1 &&
+            DEAM_IN_BOUNDS(G, k >= 0 && vk + g < (long long)G.V * G.K, SITE_BWD_TABLE, vk + g)) {
+            const InPlane ip = inplane_at(__ldg(&G.ip4[vk + g]), __ldg(&G.ipL[vk + g]));
+            const float pf = ip.axis ? fiy : fix, qf = ip.axis ? fix : fiy;
+            const float fq = __fmaf_rn(pf, ip.bq, ip.aq);
+            const float jq = floorf(fq);
+            const float aq = fq - jq;
+            float wq = 0.f;
+            if (jq == qf) wq = 1.f - aq;
+            else if (jq == qf - 1.f) wq = aq;
+            y.c[g] = ip.Lxy * wq;
+            y.t[g] = ray_t(ip, pf);
+            if (wq != 0.f) {
+                tmin = fminf(tmin, y.t[g]);
+                tmax = fmaxf(tmax, y.t[g]);
+            }
         }
     }
 }
 
-template <bool FOUR, int SLAB, int NT>
-__device__ __forceinline__ void slot_add2(float4* acc, int s, int tid, float wa, const float4& Pa, float wb,
-                                          const float4& Pb) {
-    if (s >= 0 && s < SLAB) {
-        float4& a = acc[s * NT + tid];
-        a.x = fmaf(wb, Pb.x, fmaf(wa, Pa.x, a.x));
-        a.y = fmaf(wb, Pb.y, fmaf(wa, Pa.y, a.y));
-        if (FOUR) {
-            a.z = fmaf(wb, Pb.z, fmaf(wa, Pa.z, a.z));
-            a.w = fmaf(wb, Pb.w, fmaf(wa, Pa.w, a.w));
-        }
-    }
+template <int MODE, int G_>
+__device__ __forceinline__ void fetch_rays(const Geo& G, const BwdArgs& A, const Rays<G_>& y, long long i,
+                                           Sums<MODE == BWD_UPDATE> (&P)[G_]) {
+#pragma unroll
+    for (int g = 0; g < G_; ++g)
+        if (y.c[g] != 0.f && DEAM_IN_BOUNDS(G, i + g < (long long)G.V * G.R * G.K, SITE_BWD_RAY, i + g))
+            P[g] = ray_data<MODE>(A, i + g);
 }
 
-// Rows of two rays of consecutive views at one column.  Their samples of a row
-// lie within a few hundredths of a slice of each other, so they nearly always
-// fall in the same slot pair: one read-modify-write of each slot serves both.
-template <int MODE, int SLAB, int NT>
-__device__ __forceinline__ void rows_pair(const Geo& G, const BwdArgs& A, float4* acc, int tid, int z0,
-                                          const ColRay& a, const ColRay& b) {
-    constexpr bool FOUR = MODE == BWD_UPDATE;
-    const int r0 = min(a.r0, b.r0), r1 = max(a.r1, b.r1);
-    // not unrolled: within the 64 registers of the 8-blocks-per-SM bound an
-    // unrolled body spills (measured 3 % slower at 512^2 x 64)
-#pragma unroll 1
-    for (int r = r0; r <= r1; ++r) {
-        const float4 Pa = ray_payload<MODE>(A, a.pb + (long long)r * G.K);
-        const float4 Pb = ray_payload<MODE>(A, b.pb + (long long)r * G.K);
-        const float om = row_omega(G, r);
-        const float fza = row_fz(a.sz, om, a.tp), fzb = row_fz(b.sz, om, b.tp);
-        const float jza = floorf(fza), jzb = floorf(fzb);
-        const float aza = fza - jza, azb = fzb - jzb;
-        const int sa = (int)jza - z0, sb = (int)jzb - z0;
-        const float rf = MODE == BWD_ADJOINT ? __ldg(&G.row[r]).y : 1.f;
-        const float wa = a.Lq * rf, wb = b.Lq * rf;
-        const float w1a = wa * aza, w0a = wa - w1a;
-        const float w1b = wb * azb, w0b = wb - w1b;
-        if (sa == sb) {
-            slot_add2<FOUR, SLAB, NT>(acc, sa, tid, w0a, Pa, w0b, Pb);
-            slot_add2<FOUR, SLAB, NT>(acc, sa + 1, tid, w1a, Pa, w1b, Pb);
-        } else {
-            slot_add<FOUR, SLAB, NT>(acc, sa, tid, w0a, Pa);
-            slot_add<FOUR, SLAB, NT>(acc, sa + 1, tid, w1a, Pa);
-            slot_add<FOUR, SLAB, NT>(acc, sb, tid, w0b, Pb);
-            slot_add<FOUR, SLAB, NT>(acc, sb + 1, tid, w1b, Pb);
-        }
-    }
+// A sample a above a slice (0 <= a < 1), times c: into that slice's sums lo and
+// the next one's hi.
+template <bool FOUR>
+__device__ __forceinline__ void add_sample(Sums<FOUR>& lo, Sums<FOUR>& hi, float a, float c, const Sums<FOUR>& P) {
+    const float w1 = c * a, w0 = c - w1;
+    add_scaled<FOUR>(lo, dup2(w0), P);
+    add_scaled<FOUR>(hi, dup2(w1), P);
 }
 
-// One (column tile, z-slab) of the gather backprojection: the work of one block.
-template <int MODE, int SLAB, int TX, int TY>
-__device__ __forceinline__ void bwd_tile(const Geo& G, const BwdArgs& A, float4* acc, int bx, int by, int slab) {
+// One (column tile, z-slab) of the gather backprojection: the work of one block
+// of VS groups of TX x TY threads.  Each group takes every VS-th eight views;
+// their sums are added in a fixed order (deterministic).
+template <int MODE, int SLAB, int TX, int TY, int VS>
+__device__ __forceinline__ void bwd_tile(const Geo& G, const BwdArgs& A, Sums<MODE == BWD_UPDATE>* smem, int bx, int by,
+                                         int slab) {
     // MODE: BWD_ADJOINT (A^T of two-component ray data), BWD_UPDATE (payload ->
     // b~, delta -> c-step), BWD_GRADIENT (payload -> delta = b^ - b~ = dF/dc)
     constexpr bool FOUR = MODE == BWD_UPDATE;
     constexpr int NT = TX * TY;
-    const int tid = threadIdx.x;
-    const int ix = bx * TX + (tid % TX);
-    const int iy = by * TY + (tid / TX);
-    if (ix >= G.nx || iy >= G.ny) return;  // no block-wide synchronisation below
+    static_assert(TX % 8 == 0 && TY % 4 == 0, "warps own 8 x 4 columns");
+    // a warp's 32 columns are an 8 x 4 patch: they see nearly the same ray
+    // parameter, so their rows fall between the same slices at nearly the same turn
+    const int tid = threadIdx.x % NT, group = threadIdx.x / NT;
+    const int warp = tid >> 5, lane = tid & 31;
+    const int px0 = bx * TX + (warp % (TX / 8)) * 8, py0 = by * TY + (warp / (TX / 8)) * 4;  // the warp's patch
+    // lanes in 4 x 2 blocks of columns: the eight lanes of a 128-byte wavefront
+    // read few distinct channels whatever the view's direction
+    const int lx = (lane & 3) + ((lane >> 1) & 4), ly = ((lane >> 2) & 1) + ((lane >> 3) & 2);
+    const int ix = px0 + lx, iy = py0 + ly;
+    const bool inside = ix < G.nx && iy < G.ny;
     const int z0 = slab * SLAB;
+    constexpr int G_ = kRaysPerView;
+    Sums<FOUR>* acc = smem + group * (SLAB + 2) * NT + tid;  // slot s (slice z0 - 1 + s) at acc[s * NT]
 #pragma unroll
-    for (int s = 0; s < SLAB; ++s) acc[s * NT + tid] = make_float4(0.f, 0.f, 0.f, 0.f);
+    for (int s = 0; s < SLAB + 2; ++s) acc[s * NT] = Sums<FOUR>{};
     // views that can reach this column tile's slab (host-computed per tile)
     const int2 vrange =
         __ldg(&A.slab_views[((long long)slab * ((G.ny + TY - 1) / TY) + by) * ((G.nx + TX - 1) / TX) + bx]);
     const float fix = (float)ix, fiy = (float)iy;
     const float zlo = (float)(z0 - 1), zhi = (float)(z0 + SLAB);
-    if constexpr (SLAB != 8) {
-        // views in pairs (v, v + 1): the j-th channel of one with the j-th of the other
-        for (int v = vrange.x; v <= vrange.y; v += 2) {
-            int ka0, ka1, kb0 = 0, kb1 = -1;
-            float sza, szb = 0.f;
-            view_window(G, v, fix, fiy, ka0, ka1, sza);
-            if (v + 1 <= vrange.y) view_window(G, v + 1, fix, fiy, kb0, kb1, szb);
-            const int nj = max(ka1 - ka0, kb1 - kb0) + 1;
-            for (int j = 0; j < nj; ++j) {
-                ColRay a = no_ray(), b = no_ray();
-                if (ka0 + j <= ka1) {
-                    const long long i = (long long)v * G.K + ka0 + j;
-                    a = col_ray(G, v, ka0 + j, __ldg(&G.ip4[i]), __ldg(&G.ipL[i]), ix, iy, sza, zlo, zhi);
-                }
-                if (kb0 + j <= kb1) {
-                    const long long i = (long long)(v + 1) * G.K + kb0 + j;
-                    b = col_ray(G, v + 1, kb0 + j, __ldg(&G.ip4[i]), __ldg(&G.ipL[i]), ix, iy, szb, zlo, zhi);
-                }
-                if (a.Lq == 0.f && b.Lq == 0.f) continue;
-                // a missing partner: the other ray with zero weight (same slots, same loads)
-                if (a.Lq == 0.f) {
-                    a = b;
-                    a.Lq = 0.f;
-                }
-                if (b.Lq == 0.f) {
-                    b = a;
-                    b.Lq = 0.f;
-                }
-                rows_pair<MODE, SLAB, NT>(G, A, acc, tid, z0, a, b);
-            }
+    // the patch's corners (inside the image) and the lane's place between them
+    const int ex = min(7, max(G.nx - 1 - px0, 0)), ey = min(3, max(G.ny - 1 - py0, 0));
+    const float wx = __fdividef((float)lx, (float)max(ex, 1)), wy = __fdividef((float)ly, (float)max(ey, 1));
+    const float cx = (float)(px0 + ((lane & 1) ? ex : 0)), cy = (float)(py0 + ((lane & 2) ? ey : 0));
+    for (int vb = vrange.x + 8 * group; vb <= vrange.y; vb += 8 * VS) {
+        // eight views at a time: every lane looks at one view from one corner of
+        // the warp's patch (a window costs as much as a row of samples)
+        const CornerWindow C = corner_window(G, min(vb + (lane >> 2), vrange.y), cx, cy, zlo, zhi);
+        float hw = C.hw, lo = C.lo, hi = C.hi;
+#pragma unroll
+        for (int o = 1; o < 4; o <<= 1) {
+            hw = fmaxf(hw, __shfl_xor_sync(0xffffffffu, hw, o));
+            lo = fminf(lo, __shfl_xor_sync(0xffffffffu, lo, o));
+            hi = fmaxf(hi, __shfl_xor_sync(0xffffffffu, hi, o));
         }
-    } else {
-        for (int v = vrange.x; v <= vrange.y; ++v) {
-            int k0, k1;
-            float sz;
-            view_window(G, v, fix, fiy, k0, k1, sz);
-            const long long vbase = (long long)v * G.K;
-            float4 na = make_float4(0.f, 0.f, 0.f, 0.f);
-            float nl = 1.f;
-            if (k0 <= k1) {
-                na = __ldg(&G.ip4[vbase + k0]);
-                nl = __ldg(&G.ipL[vbase + k0]);
+        lo = fminf(lo, __shfl_xor_sync(0xffffffffu, lo, 4));  // both views of a pair
+        hi = fmaxf(hi, __shfl_xor_sync(0xffffffffu, hi, 4));
+        const int row0 = max(0, __float2int_ru(fminf(lo, (float)G.R)));
+        const int row1 = min(G.R - 1, __float2int_rd(fmaxf(fminf(hi, (float)G.R), -1.f)));
+        // Views in pairs: their samples of a row lie within a few hundredths of a
+        // slice of each other, so nearly always all between the same two slices
+        // (one read and write of their sums serves the rays of both)
+        const int nv = min(8, vrange.y - vb + 1);
+        for (int w = 0; w < nv; w += 2) {
+            const int v = vb + w;
+            const int r0 = __shfl_sync(0xffffffffu, row0, 4 * w), r1 = __shfl_sync(0xffffffffu, row1, 4 * w);
+            float u[2], h[2];
+#pragma unroll
+            for (int q = 0; q < 2; ++q) {
+                const int l = 4 * (w + q);
+                const float a = __shfl_sync(0xffffffffu, C.u, l), b = __shfl_sync(0xffffffffu, C.u, l + 1);
+                const float c = __shfl_sync(0xffffffffu, C.u, l + 2), d = __shfl_sync(0xffffffffu, C.u, l + 3);
+                const float lu = fmaf(wx, b - a, a), hu = fmaf(wx, d - c, c);
+                u[q] = fmaf(wy, hu - lu, lu);
+                h[q] = __shfl_sync(0xffffffffu, hw, l);
             }
-            for (int k = k0; k <= k1; ++k) {
-                const InPlane ip = inplane_at(na, nl);
-                if (k < k1) {  // prefetch the next channel's parameters
-                    na = __ldg(&G.ip4[vbase + k + 1]);
-                    nl = __ldg(&G.ipL[vbase + k + 1]);
-                }
-                const int p = ip.axis ? iy : ix;
-                const int q = ip.axis ? ix : iy;
-                const float pf = (float)p;
-                const float fq = __fmaf_rn(pf, ip.bq, ip.aq);
-                const float jq = floorf(fq);
-                const float aq = fq - jq;
-                float wq;
-                if (jq == (float)q) wq = 1.f - aq;
-                else if (jq == (float)(q - 1)) wq = aq;
-                else continue;
-                if (wq == 0.f) continue;
-                const float tp = ray_t(ip, pf);  // ray parameter at plane p
-                int r0 = 0, r1 = G.R - 1;
-                if (G.R > 1) {
-                    // fz(r) = sigma_z + t (omega0 + r domega): rows whose sample can
-                    // land in [z0 - 1, z0 + SLAB).  Solved in FP32 with the fast
-                    // reciprocal (within ~1e-6 rows of the rounded samples); a
-                    // 0.02-row margin keeps every contributing row, and the exact
-                    // per-row slot test below decides.
-                    const float slope = tp * G.domega;
-                    if (fabsf(slope) > 1e-20f) {
-                        const float inv = __fdividef(1.f, slope);
-                        const float base = fmaf(tp, G.omega0, sz);
-                        const float ra = (zlo - base) * inv, rb = (zhi - base) * inv;
-                        const float lo = fminf(fmaxf(fminf(ra, rb), -4.f), (float)G.R + 4.f);
-                        const float hi = fminf(fmaxf(fmaxf(ra, rb), -4.f), (float)G.R + 4.f);
-                        r0 = max(0, (int)floorf(lo - 0.02f));
-                        r1 = min(G.R - 1, (int)ceilf(hi + 0.02f));
-                    }
-                }
-                const float Lq = ip.Lxy * wq;
-                // two or more rows fall in one slice, so consecutive rows add to the
-                // same slot pair: keep it in registers (plo: slot ls, phi: slot
-                // ls + 1) and write shared memory when the slot moves on
-                float4 plo = make_float4(0.f, 0.f, 0.f, 0.f), phi = plo;
-                int ls = -1000;
-                // ray data [V][R][K]: a warp's columns read neighbouring channels of a row
-                const long long pb = vbase * G.R + k;
-                if (!DEAM_IN_BOUNDS(G, pb + (long long)r1 * G.K < (long long)G.V * G.R * G.K, SITE_BWD_RAY,
-                                    pb + (long long)r1 * G.K))
-                    continue;
-    #pragma unroll 4
+            if (r0 > r1) continue;  // no row of these views reaches the slab
+            if (!inside) continue;
+            const bool second = w + 1 < nv;
+            const int ka0 = max(0, __float2int_ru(fmaxf(u[0] - h[0], -1.f)));
+            const int ka1 = min(G.K - 1, __float2int_rd(fminf(u[0] + h[0], (float)G.K)));
+            const int kb0 = max(0, __float2int_ru(fmaxf(u[1] - h[1], -1.f)));
+            const int kb1 = second ? min(G.K - 1, __float2int_rd(fminf(u[1] + h[1], (float)G.K))) : kb0 - 1;
+            const float sza = __ldg(&G.view_z[v]), szb = __ldg(&G.view_z[second ? v + 1 : v]);
+            const int n = max(ka1 - ka0, kb1 - kb0);
+            for (int j = 0; j <= n; j += G_) {
+                Rays<G_> a, b;
+                float ta0 = INFINITY, ta1 = 0.f, tb0 = INFINITY, tb1 = 0.f;
+                load_rays<G_>(G, a, v, ka0 + j, ka1, fix, fiy, ta0, ta1);
+                load_rays<G_>(G, b, v + 1, kb0 + j, kb1, fix, fiy, tb0, tb1);
+                if (ta1 == 0.f && tb1 == 0.f) continue;
+                long long i = ((long long)v * G.R + r0) * G.K + j;
+                const long long next_view = (long long)G.R * G.K;
+                Sums<FOUR> P[G_], Q[G_];
+#pragma unroll
+                for (int g = 0; g < G_; ++g) P[g] = Q[g] = Sums<FOUR>{};
+                float rf = (float)r0;
+#pragma unroll 1
                 for (int r = r0; r <= r1; ++r) {
-                    float4 Pv;
-                    if (MODE == BWD_ADJOINT) {
-                        const float2 t = __ldg(&A.rays2[pb + (long long)r * G.K]);
-                        Pv = make_float4(t.x, t.y, 0.f, 0.f);
-                    } else {
-                        Pv = __ldg(&A.payload[pb + (long long)r * G.K]);
-                        if (MODE == BWD_GRADIENT) Pv = make_float4(Pv.z, Pv.w, 0.f, 0.f);
+                    fetch_rays<MODE, G_>(G, A, a, i + ka0, P);
+                    fetch_rays<MODE, G_>(G, A, b, i + next_view + kb0, Q);
+                    const float om = __fmaf_rn(rf, G.domega, G.omega0);
+                    const float rowf = MODE == BWD_ADJOINT ? __ldg(&G.row[r]).y : 1.f;
+                    rf += 1.f;
+                    i += G.K;
+                    // lowest and highest sample of the row
+                    const float za0 = row_fz(sza, om, ta0), za1 = row_fz(sza, om, ta1);
+                    const float zb0 = row_fz(szb, om, tb0), zb1 = row_fz(szb, om, tb1);
+                    float zmin = INFINITY, zmax = -INFINITY;
+                    if (ta1 != 0.f) {
+                        zmin = fminf(za0, za1);
+                        zmax = fmaxf(za0, za1);
                     }
-                    const float fz = row_fz(sz, row_omega(G, r), tp);
-                    const float jz = floorf(fz);
-                    const float az = fz - jz;
-                    const int sl = (int)jz - z0;
-                    // the payload carries h's row length factor already (folded by
-                    // the forward kernel); A^T of caller data applies it here
-                    const float w = MODE == BWD_ADJOINT ? Lq * __ldg(&G.row[r]).y : Lq;
-                    const float w1 = w * az, w0 = w - w1;
-                    if (sl != ls) {   // slots rise with r: flush the slot that is complete
-                        pend_flush<FOUR, SLAB, NT>(acc, ls, tid, plo);
-                        if (sl == ls + 1) {
-                            plo = phi;
-                        } else {
-                            pend_flush<FOUR, SLAB, NT>(acc, ls + 1, tid, phi);
-                            plo = make_float4(0.f, 0.f, 0.f, 0.f);
+                    if (tb1 != 0.f) {
+                        zmin = fminf(zmin, fminf(zb0, zb1));
+                        zmax = fmaxf(zmax, fmaxf(zb0, zb1));
+                    }
+                    const float f = floorf(zmin);
+                    const int slot = (int)f - (z0 - 1);
+                    if (zmax < f + 1.f) {
+                        if (slot < 0 || slot > SLAB) continue;
+                        Sums<FOUR> lo = acc[slot * NT], hi = acc[(slot + 1) * NT];
+#pragma unroll
+                        for (int g = 0; g < G_; ++g) {
+                            add_sample<FOUR>(lo, hi, row_fz(sza, om, a.t[g]) - f, a.c[g] * rowf, P[g]);
+                            add_sample<FOUR>(lo, hi, row_fz(szb, om, b.t[g]) - f, b.c[g] * rowf, Q[g]);
                         }
-                        phi = make_float4(0.f, 0.f, 0.f, 0.f);
-                        ls = sl;
-                    }
-                    plo.x = fmaf(w0, Pv.x, plo.x);
-                    plo.y = fmaf(w0, Pv.y, plo.y);
-                    phi.x = fmaf(w1, Pv.x, phi.x);
-                    phi.y = fmaf(w1, Pv.y, phi.y);
-                    if (FOUR) {
-                        plo.z = fmaf(w0, Pv.z, plo.z);
-                        plo.w = fmaf(w0, Pv.w, plo.w);
-                        phi.z = fmaf(w1, Pv.z, phi.z);
-                        phi.w = fmaf(w1, Pv.w, phi.w);
+                        acc[slot * NT] = lo;
+                        acc[(slot + 1) * NT] = hi;
+                    } else {
+#pragma unroll 1
+                        for (int s = max(slot, 0); s <= SLAB; ++s) {
+                            const float fs = (float)(z0 - 1 + s);
+                            if (zmax < fs) break;
+                            Sums<FOUR> lo = acc[s * NT], hi = acc[(s + 1) * NT];
+#pragma unroll
+                            for (int g = 0; g < G_; ++g) {
+                                const float x = row_fz(sza, om, a.t[g]) - fs, y = row_fz(szb, om, b.t[g]) - fs;
+                                if (x >= 0.f && x < 1.f) add_sample<FOUR>(lo, hi, x, a.c[g] * rowf, P[g]);
+                                if (y >= 0.f && y < 1.f) add_sample<FOUR>(lo, hi, y, b.c[g] * rowf, Q[g]);
+                            }
+                            acc[s * NT] = lo;
+                            acc[(s + 1) * NT] = hi;
+                        }
                     }
                 }
-                pend_flush<FOUR, SLAB, NT>(acc, ls, tid, plo);
-                pend_flush<FOUR, SLAB, NT>(acc, ls + 1, tid, phi);
             }
         }
+        __syncwarp();
     }
-
+    if constexpr (VS > 1) __syncthreads();
+    if (!inside) return;
     unsigned long long skipped = 0;
-    for (int s = 0; s < SLAB; ++s) {
+#pragma unroll 1
+    for (int s = group; s < SLAB; s += VS) {  // the groups share out the slices
         const int iz = z0 + s;
         if (iz >= G.nz) break;
-        const float4 a = acc[s * NT + tid];
+        Sums<FOUR> sum = smem[(s + 1) * NT + tid];
+#pragma unroll
+        for (int g = 1; g < VS; ++g) add_to<FOUR>(sum, smem[(g * (SLAB + 2) + s + 1) * NT + tid]);
+        const float2 lo = unpack2(sum.a);
+        float4 a = make_float4(lo.x, lo.y, 0.f, 0.f);
+        if constexpr (FOUR) {
+            const float2 hi = unpack2(sum.b);
+            a.z = hi.x;
+            a.w = hi.y;
+        }
         const long long vi = ((long long)iz * G.ny + iy) * G.nx + ix;
         if (!DEAM_IN_BOUNDS(G, vi < (long long)G.nx * G.ny * G.nz, SITE_BWD_IMAGE, vi)) break;
         if (!FOUR) {  // A^T y, or the gradient delta_i
@@ -399,30 +411,32 @@ __device__ __forceinline__ void bwd_tile(const Geo& G, const BwdArgs& A, float4*
     if (FOUR && skipped) atomicAdd(A.skipped, skipped);
 }
 
+// Column tile of a block of VS view groups
+template <int VS>
+struct BwdTile {
+    static constexpr int X = bwd_tile_x(VS), Y = bwd_tile_y(VS);
+    static_assert(X * Y * VS == kBwdThreads, "view groups x columns fill the block");
+};
 
-
-// At most 64 registers a thread: 8 blocks per SM (shared memory allows it up
-// to kDeepSlab slices); more resident warps hide the gathers' latency.
-template <int MODE, int SLAB>
-__global__ void __launch_bounds__(kBwdThreads, 8) bwd_kernel(const Geo G, const BwdArgs A) {
-    __shared__ float4 acc[SLAB * kBwdThreads];
-    const int ntx = (G.nx + kTileX - 1) / kTileX, nty = (G.ny + kTileY - 1) / kTileY;
+template <int MODE, int SLAB, int VS>
+__global__ void __launch_bounds__(kBwdThreads, 5) bwd_kernel(const Geo G, const BwdArgs A) {
+    constexpr int TX = BwdTile<VS>::X, TY = BwdTile<VS>::Y;
+    __shared__ Sums<MODE == BWD_UPDATE> acc[(SLAB + 2) * kBwdThreads];
+    const int ntx = (G.nx + TX - 1) / TX, nty = (G.ny + TY - 1) / TY;
     int b = blockIdx.x;
     const int bx = b % ntx;
     b /= ntx;
     const int by = b % nty;
-    bwd_tile<MODE, SLAB, kTileX, kTileY>(G, A, acc, bx, by, b / nty);
+    bwd_tile<MODE, SLAB, TX, TY, VS>(G, A, acc, bx, by, b / nty);
 }
 
 // Batched scans: one persistent launch walks the column tiles x slabs of every
 // scan of a slab class; each work item finds its scan by binary search in the
 // prefix sums of tile counts.
-// (the backprojection keeps the scan's descriptors in registers: staging them
-// in shared memory was measured slower for this kernel; bounded to the
-// single-scan kernel's 6 blocks/SM, which it now meets without spilling)
+// (the scan's descriptors are held in registers, hence one block per SM less)
 template <int SLAB, int TX, int TY>
-__global__ void __launch_bounds__(TX* TY, 6) bwd_batch_kernel(const BatchDesc B) {
-    __shared__ float4 acc[SLAB * TX * TY];
+__global__ void __launch_bounds__(TX* TY, 4) bwd_batch_kernel(const BatchDesc B) {
+    __shared__ Sums<true> acc[(SLAB + 2) * TX * TY];
     const long long total = __ldg(&B.btile_off[B.n]);
     for (long long t = blockIdx.x; t < total; t += gridDim.x) {
         const int i = find_scan(B.btile_off, B.n, t);
@@ -433,33 +447,32 @@ __global__ void __launch_bounds__(TX* TY, 6) bwd_batch_kernel(const BatchDesc B)
         const int bx = (int)(lt % ntx);
         lt /= ntx;
         const int by = (int)(lt % nty);
-        bwd_tile<BWD_UPDATE, SLAB, TX, TY>(G, A, acc, bx, by, (int)(lt / nty));
+        bwd_tile<BWD_UPDATE, SLAB, TX, TY, 1>(G, A, acc, bx, by, (int)(lt / nty));
     }
 }
 
-
-cudaError_t launch_backward(int mode, int slab, const Geo& G, const BwdArgs& A, cudaStream_t s) {
-    const int ntx = (G.nx + kTileX - 1) / kTileX, nty = (G.ny + kTileY - 1) / kTileY;
-    const int nsl = (G.nz + slab - 1) / slab;
-    const int blocks = ntx * nty * nsl;
-#define DEAM_BWD(M, SL) bwd_kernel<M, SL><<<blocks, kBwdThreads, 0, s>>>(G, A)
-    if (slab == 2) {
-        if (mode == BWD_UPDATE) DEAM_BWD(BWD_UPDATE, 2);
-        else if (mode == BWD_GRADIENT) DEAM_BWD(BWD_GRADIENT, 2);
-        else DEAM_BWD(BWD_ADJOINT, 2);
-    } else if (slab == 8) {
-        if (mode == BWD_UPDATE) DEAM_BWD(BWD_UPDATE, 8);
-        else if (mode == BWD_GRADIENT) DEAM_BWD(BWD_GRADIENT, 8);
-        else DEAM_BWD(BWD_ADJOINT, 8);
-    } else if (slab == kDeepSlab) {
-        if (mode == BWD_UPDATE) DEAM_BWD(BWD_UPDATE, kDeepSlab);
-        else if (mode == BWD_GRADIENT) DEAM_BWD(BWD_GRADIENT, kDeepSlab);
-        else DEAM_BWD(BWD_ADJOINT, kDeepSlab);
-    } else {
-        return cudaErrorInvalidValue;
-    }
-#undef DEAM_BWD
+template <int SLAB, int VS>
+static cudaError_t launch_bwd(int mode, const Geo& G, const BwdArgs& A, cudaStream_t s) {
+    constexpr int TX = BwdTile<VS>::X, TY = BwdTile<VS>::Y;
+    const int blocks = ((G.nx + TX - 1) / TX) * ((G.ny + TY - 1) / TY) * ((G.nz + SLAB - 1) / SLAB);
+    if (mode == BWD_UPDATE) bwd_kernel<BWD_UPDATE, SLAB, VS><<<blocks, kBwdThreads, 0, s>>>(G, A);
+    else if (mode == BWD_GRADIENT) bwd_kernel<BWD_GRADIENT, SLAB, VS><<<blocks, kBwdThreads, 0, s>>>(G, A);
+    else bwd_kernel<BWD_ADJOINT, SLAB, VS><<<blocks, kBwdThreads, 0, s>>>(G, A);
     return cudaGetLastError();
+}
+
+cudaError_t launch_backward(int mode, const BwdPlan& P, const Geo& G, const BwdArgs& A, cudaStream_t s) {
+#define DEAM_BWD(SL, VS) \
+    if (P.slab == SL && P.vs == VS) return launch_bwd<SL, VS>(mode, G, A, s);
+    DEAM_BWD(2, 4)
+    DEAM_BWD(kMidSlab, 1)
+    DEAM_BWD(kMidSlab, 2)
+    DEAM_BWD(kMidSlab, 4)
+    DEAM_BWD(kDeepSlab, 1)
+    DEAM_BWD(kDeepSlab, 2)
+    DEAM_BWD(kDeepSlab, 4)
+#undef DEAM_BWD
+    return cudaErrorInvalidValue;
 }
 
 long long backward_tiles(int shape, const Geo& G) {

@@ -247,7 +247,7 @@ static int record_iteration(deam_batch* b, float* const* c, int plan) {
             B.clamp_nonneg = x->clamp;
             B.skipped = x->skipped;
             deam::set_penalty_args(x, B);
-            if (e == cudaSuccess) e = deam::launch_backward(deam::BWD_UPDATE, x->slab, x->G, B, q);
+            if (e == cudaSuccess) e = deam::launch_backward(deam::BWD_UPDATE, x->bwd, x->G, B, q);
             if (e == cudaSuccess && B.sums) e = deam::launch_reg_update(x->G, B, q);
             if (e == cudaSuccess) e = cudaEventRecord(b->join[i], q);
             if (e == cudaSuccess) e = cudaStreamWaitEvent(s, b->join[i], 0);

@@ -25,7 +25,8 @@ struct deam_ctx {
     bool has_data = false, mask_set = false, failed = false;
     int batch_refs = 0;                // live batches holding this context (deam_destroy refuses)
     long long nrays = 0, nvox = 0, skipped_last = 0;
-    int n_fwd_blocks = 0, n_slabs = 0, slab = 16;
+    int n_fwd_blocks = 0;
+    deam::BwdPlan bwd;                 // how the backprojection splits its work
     // device buffers
     float4* view4 = nullptr;
     float* view_z = nullptr;

@@ -16,8 +16,6 @@ constexpr int kTileK = 32;        // forward ray tile: channels (one warp) ...
 constexpr int kTileR = 4;         // ... x rows ...
 constexpr int kTileV = 2;         // ... x views
 constexpr int kFwdThreads = kTileK * kTileR * kTileV;  // rays per forward block (256)
-constexpr int kTileX = 16;        // backprojector column tile (x)
-constexpr int kTileY = 8;         // backprojector column tile (y)
 
 // Geometry in voxel-index units, as read by both projector directions.  Every
 // per-ray quantity is derived from these tables by ray_inplane()/row terms with
@@ -37,6 +35,7 @@ struct Geo {
     float omega0, domega;    // omega_r = omega0 + r domega (row_omega)
     float chan_c0, inv_dgamma;  // channel coordinate = gamma / dgamma + chan_c0
     float vox_reach_mm;      // max(dx, dy): reach of a voxel's bilinear footprint in-plane
+    float inv_sdd;           // 1 / sdd: in-plane distance from the source -> ray parameter t
     unsigned int* fault;     // [2] bounds-checked builds: first failing site and index (else unused)
 };
 
@@ -202,20 +201,40 @@ constexpr int kBwdShapes[kNumBwdShapes][3] = {{2, 16, 8}, {2, 32, 4}, {8, 16, 8}
                                               {8, 32, 4}, {16, 16, 8}, {16, 32, 4}};  // (slab, tx, ty)
 // Slab class of the gather backprojection for a scan: 2 for one or two
 // slices, 8 when a detector row covers at most 2/3 of a slice (several rows
-// per slot), else 16.  The batched persistent launches use the class as their
-// slab depth; a single-scan context runs class 16 as kDeepSlab slices.
+// per slice), else 16.  The batched persistent launches use the class as their
+// slab depth; a single-scan context runs its own plan (bwd_plan).
 inline int pick_slab(int nz, int n_rows, double dz, double row_pitch, double sid, double sdd) {
     if (nz <= 2) return 2;
     return (n_rows == 1 || dz >= 1.5 * row_pitch * sid / sdd) ? 8 : 16;
 }
-// Slab depth a single-scan context runs for the deep class (16): 13 slices.
-// The accumulators of a 128-thread block then take 26 KB of shared memory, so
-// with at most 64 registers a thread 8 blocks (32 warps) fit on an SM instead
-// of 6: the gather is latency-bound at 6 (measured at 512^2 x 64: 16 slices at
-// 6 blocks/SM 203.8 ms, 12 at 7 blocks 193.0 ms, 11 at 8 blocks 189.7 ms).
-// The batched persistent launches keep their own shapes (kBwdShapes).
-constexpr int kDeepSlab = 13;
-inline int context_slab(int slab_class) { return slab_class == 16 ? kDeepSlab : slab_class; }
+// How a single-scan context backprojects: z-slabs of `slab` slices, and the views
+// of a column shared out over `vs` warps (whose sums are added at the end).
+//   slab: a deep slab costs less set-up per sample (a slab is visited by the views
+//   of slab + rows covered), a shallow one leaves more of the 256 KB to L1.  16
+//   against 13 slices, deep class: 18.7 / 19.8 ms at 384^2 x 48, 11.5 / 12.5 ms at
+//   256^2 x 16 x 1440 views, 22.9 / 23.1 ms on a rotation of 512^2 x 64.  11
+//   against 16 slices with several rows per slice: 8.5 / 9.8 ms on a rotation of
+//   256^2 x 32 x 672 channels.
+//   vs: 5 blocks of 4 warps run on an SM; below 8 rounds of the GPU the views are
+//   split so that the last, part-filled round weighs less: 4 warps against 1
+//   11.8 -> 9.9 ms (256^2 x 16: 2048 warps of columns), 11.7 -> 8.5 ms (256^2 x 32);
+//   2 against 1 19.4 -> 18.8 ms (384^2 x 48: 13,824); at 512^2 x 64 (32,768) 1 is
+//   as fast as 2 and 3 % faster than 4.
+struct BwdPlan {
+    int slab = 2, vs = 4;
+};
+constexpr int kMidSlab = 11, kDeepSlab = 16;
+constexpr int bwd_tile_x(int vs) { return vs == 1 ? 16 : 8; }
+constexpr int bwd_tile_y(int vs) { return vs == 4 ? 4 : 8; }
+inline BwdPlan bwd_plan(int nx, int ny, int nz, int slab_class, int sms) {
+    BwdPlan p;
+    if (slab_class == 2) return p;
+    p.slab = slab_class == 8 ? kMidSlab : kDeepSlab;
+    const long long warps = (long long)((nx + 7) / 8) * ((ny + 3) / 4) * ((nz + p.slab - 1) / p.slab);
+    const long long round = 20LL * sms;
+    p.vs = warps >= 8 * round ? 1 : warps >= 4 * round ? 2 : 4;
+    return p;
+}
 long long forward_tiles(int shape, const Geo& G);
 long long backward_tiles(int shape, const Geo& G);
 int forward_batch_blocks_per_sm(int shape);
@@ -233,7 +252,7 @@ cudaError_t launch_layout(const float2* c, const float* m, int ones, float4* vol
 int forward_blocks_per_sm();
 cudaError_t launch_forward(int mode, const Geo& G, const Spec& S, const FwdArgs& A, int n_blocks,
                            cudaStream_t s);
-cudaError_t launch_backward(int mode, int slab, const Geo& G, const BwdArgs& A, cudaStream_t s);
+cudaError_t launch_backward(int mode, const BwdPlan& P, const Geo& G, const BwdArgs& A, cudaStream_t s);
 cudaError_t launch_sum_partials(const double* partial, int n, double* out, int do_max, cudaStream_t s);
 cudaError_t launch_clamp_copy(const float* d, float* dt, long long n, cudaStream_t s);
 cudaError_t launch_mask_bits(uint8_t* m, long long n, int per_spectrum, cudaStream_t s);
