@@ -16,7 +16,7 @@ LIB = os.path.join(HERE, "libdeam.so")
 # an out-of-range index and the entry point returns DEAM_ERR_ARG
 LIB_CHECKED = os.path.join(HERE, "libdeam_checked.so")
 SOURCES = ["deam_kernels.cu", "deam_backproject.cu", "deam_api.cu", "deam_batch.cu", "deam_noalloc.cu", "deam_mar.cu"]
-HEADERS = ["deam_internal.h", "deam_epilogue.cuh", "deam_ctx.h", os.path.join("..", "..", "include", "deam.h")]
+HEADERS = ["deam_internal.h", "deam_epilogue.cuh", "deam_pair.cuh", "deam_ctx.h", os.path.join("..", "..", "include", "deam.h")]
 ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]
 FLAGS = ["-O3", "-lineinfo", "-std=c++17", "-Xcompiler", "-fPIC", "-I", os.path.join(ROOT, "include")]
 

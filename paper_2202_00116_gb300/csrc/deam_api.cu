@@ -287,10 +287,6 @@ int deam_init(const deam_geometry* geom, const deam_spectra* spectra, const deam
     int sms = 152;
     cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, ctx->device);
     ctx->bwd = deam::bwd_plan(g.nx, g.ny, g.nz, deam::pick_slab(g.nz, g.n_rows, g.dz, g.row_pitch, g.sid, g.sdd), sms);
-    const long long ntiles = (long long)((g.n_channels + deam::kTileK - 1) / deam::kTileK) *
-                             ((g.n_rows + deam::kTileR - 1) / deam::kTileR) *
-                             ((g.n_views + deam::kTileV - 1) / deam::kTileV);
-    ctx->n_fwd_blocks = (int)std::min<long long>(ntiles, (long long)sms * deam::forward_blocks_per_sm());
 
     // ---- geometry tables (double on the host, rounded once to float) ----
     const double X0 = g.cx - (g.nx - 1) / 2.0 * g.dx, Y0 = g.cy - (g.ny - 1) / 2.0 * g.dy,
@@ -325,6 +321,8 @@ int deam_init(const deam_geometry* geom, const deam_spectra* spectra, const deam
     G.domega = (float)(g.row_pitch / g.dz);
     G.chan_c0 = (float)((g.n_channels - 1) / 2.0 - g.channel_offset);
     G.inv_dgamma = (float)(1.0 / g.channel_pitch);
+    G.fwd_rows = deam::forward_rows(g);
+    ctx->n_fwd_blocks = deam::forward_blocks(G, sms);
     G.vox_reach_mm = (float)(std::max(g.dx, g.dy) * 1.001);
     G.inv_sdd = (float)(1.0 / g.sdd);
 

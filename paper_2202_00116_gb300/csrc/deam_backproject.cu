@@ -7,6 +7,7 @@
 #include <math.h>
 
 #include "deam_internal.h"
+#include "deam_pair.cuh"
 
 namespace deam {
 
@@ -36,32 +37,6 @@ constexpr int kBwdThreads = 128;
 // Four at 5 blocks of 128 threads per SM; three at 6 blocks are as fast at 2.6
 // rays per view and 8 % slower at 3.5 (384^2 x 48 on 816 channels).
 constexpr int kRaysPerView = 4;
-
-typedef unsigned long long pair32;  // two FP32 values in a register pair
-
-__device__ __forceinline__ pair32 pack2(float x, float y) {
-    pair32 r;
-    asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(x), "f"(y));
-    return r;
-}
-__device__ __forceinline__ float2 unpack2(pair32 v) {
-    float2 r;
-    asm("mov.b64 {%0, %1}, %2;" : "=f"(r.x), "=f"(r.y) : "l"(v));
-    return r;
-}
-// a b + c on both halves, each rounded as fmaf rounds it
-__device__ __forceinline__ pair32 fma2(pair32 a, pair32 b, pair32 c) {
-    pair32 d;
-    asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(d) : "l"(a), "l"(b), "l"(c));
-    return d;
-}
-
-__device__ __forceinline__ pair32 add2(pair32 a, pair32 b) {
-    pair32 d;
-    asm("add.rn.f32x2 %0, %1, %2;" : "=l"(d) : "l"(a), "l"(b));
-    return d;
-}
-__device__ __forceinline__ pair32 dup2(float x) { return pack2(x, x); }
 
 // A ray's data, or the sums of a voxel: (b~_1, b~_2) and, for the c-step, also
 // (delta_1, delta_2).  The gradient carries the second pair alone, the plain

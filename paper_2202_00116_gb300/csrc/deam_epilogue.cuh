@@ -71,58 +71,95 @@ __device__ __forceinline__ T block_reduce(T v, bool is_max) {
     return v;
 }
 
-// Spectral sums of one ray for both spectra: g_j = sum_E I0_j q~, S_ij = sum_E
-// mu_i I0_j q~ with q~ = 2^(-mu'.l) (bowtie applied by the caller).  Bins are
-// summed in blocks of 8 in FP32, block partials are added with compensation.
+// The six sums of one ray over the energy bins: g_j = sum_E I0_j q~ and S_ij =
+// sum_E mu_i I0_j q~ (j = L, H), q~ = 2^(-mu'.l).
+struct RaySums {
+    float gl, gh, s1l, s2l, s1h, s2h;
+};
+
+template <bool NEED_S>
+__device__ __forceinline__ void add_bin(RaySums& p, float ex, float mu1, float mu2, float i0l, float i0h) {
+    p.gl = fmaf(i0l, ex, p.gl);
+    p.gh = fmaf(i0h, ex, p.gh);
+    if (NEED_S) {
+        const float ql = __fmul_rn(i0l, ex), qh = __fmul_rn(i0h, ex);
+        p.s1l = fmaf(mu1, ql, p.s1l);
+        p.s2l = fmaf(mu2, ql, p.s2l);
+        p.s1h = fmaf(mu1, qh, p.s1h);
+        p.s2h = fmaf(mu2, qh, p.s2h);
+    }
+}
+
+template <bool NEED_S>
+__device__ __forceinline__ void kahan_add(RaySums& s, RaySums& c, const RaySums& p) {
+    kahan_add(s.gl, c.gl, p.gl);
+    kahan_add(s.gh, c.gh, p.gh);
+    if (NEED_S) {
+        kahan_add(s.s1l, c.s1l, p.s1l);
+        kahan_add(s.s2l, c.s2l, p.s2l);
+        kahan_add(s.s1h, c.s1h, p.s1h);
+        kahan_add(s.s2h, c.s2h, p.s2h);
+    }
+}
+
+// Spectral tables in shared memory, as the sums over many rays read them: active
+// bin e at a[e] = (mu_1', mu_2', mu_1, mu_2), b[e] = (I0_L, I0_H).
+struct SpecTable {
+    float4 a[kMaxE];
+    float2 b[kMaxE];
+};
+__device__ __forceinline__ void fill_table(SpecTable& T, const Spec& S) {
+    for (int e = S.e_lo + threadIdx.x; e < S.e_hi; e += blockDim.x) {
+        T.a[e - S.e_lo] = make_float4(S.mu1l2[e], S.mu2l2[e], S.mu1[e], S.mu2[e]);
+        T.b[e - S.e_lo] = make_float2(S.i0l[e], S.i0h[e]);
+    }
+}
+
+// Spectral sums of N rays for both spectra (bowtie applied by the caller).  Bins
+// are summed in blocks of 8 in FP32, block partials are added with compensation.
 // COMP = false: plain FP32 sums, bin after bin (the uncompensated variant).
-template <bool NEED_S, bool COMP = true>
-__device__ __forceinline__ void spectral_sums(const Spec& S, float l1, float l2, float& gl, float& gh,
-                                              float& s1l, float& s2l, float& s1h, float& s2h) {
-    float cgl = 0.f, cgh = 0.f, c1l = 0.f, c2l = 0.f, c1h = 0.f, c2h = 0.f;
-    gl = gh = s1l = s2l = s1h = s2h = 0.f;
-    if constexpr (!COMP) {
-        for (int e = S.e_lo; e < S.e_hi; ++e) {
-            const float ex = ex2_approx(-fmaf(S.mu1l2[e], l1, S.mu2l2[e] * l2));
-            const float ql = S.i0l[e] * ex, qh = S.i0h[e] * ex;
-            gl += ql;
-            gh += qh;
-            if (NEED_S) {
-                s1l = fmaf(S.mu1[e], ql, s1l);
-                s2l = fmaf(S.mu2[e], ql, s2l);
-                s1h = fmaf(S.mu1[e], qh, s1h);
-                s2h = fmaf(S.mu2[e], qh, s2h);
-            }
-        }
-    } else {
-        for (int e0 = S.e_lo; e0 < S.e_hi; e0 += 8) {
-            float pgl = 0.f, pgh = 0.f, p1l = 0.f, p2l = 0.f, p1h = 0.f, p2h = 0.f;
-            const int n = min(8, S.e_hi - e0);
+// bin(e) gives the table entry of active bin e of n.
+template <bool NEED_S, bool COMP, int N, typename Bin>
+__device__ __forceinline__ void spectral_sums(int n, const float (&l1)[N], const float (&l2)[N], RaySums (&s)[N], Bin bin) {
+    RaySums c[N], p[N];
 #pragma unroll
-            for (int i = 0; i < 8; ++i) {
-                if (i < n) {
-                    const int e = e0 + i;
-                    const float ex = ex2_approx(-fmaf(S.mu1l2[e], l1, S.mu2l2[e] * l2));
-                    const float ql = S.i0l[e] * ex, qh = S.i0h[e] * ex;
-                    pgl += ql;
-                    pgh += qh;
-                    if (NEED_S) {
-                        p1l = fmaf(S.mu1[e], ql, p1l);
-                        p2l = fmaf(S.mu2[e], ql, p2l);
-                        p1h = fmaf(S.mu1[e], qh, p1h);
-                        p2h = fmaf(S.mu2[e], qh, p2h);
-                    }
-                }
-            }
-            kahan_add(gl, cgl, pgl);
-            kahan_add(gh, cgh, pgh);
-            if (NEED_S) {
-                kahan_add(s1l, c1l, p1l);
-                kahan_add(s2l, c2l, p2l);
-                kahan_add(s1h, c1h, p1h);
-                kahan_add(s2h, c2h, p2h);
-            }
+    for (int i = 0; i < N; ++i) s[i] = c[i] = RaySums{0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
+    auto one = [&](int e, RaySums(&to)[N]) {
+        float4 a;
+        float2 b;
+        bin(e, a, b);
+#pragma unroll
+        for (int i = 0; i < N; ++i) {
+            const float ex = ex2_approx(-fmaf(a.x, l1[i], a.y * l2[i]));
+            add_bin<NEED_S>(to[i], ex, a.z, a.w, b.x, b.y);
+        }
+    };
+    if constexpr (!COMP) {
+        for (int e = 0; e < n; ++e) one(e, s);
+    } else {
+        for (int e0 = 0; e0 < n; e0 += 8) {
+#pragma unroll
+            for (int i = 0; i < N; ++i) p[i] = RaySums{0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
+#pragma unroll
+            for (int j = 0; j < 8; ++j)
+                if (e0 + j < n) one(e0 + j, p);
+#pragma unroll
+            for (int i = 0; i < N; ++i) kahan_add<NEED_S>(s[i], c[i], p[i]);
         }
     }
+}
+
+// One ray, the tables read from the kernel's parameters.
+template <bool NEED_S, bool COMP = true>
+__device__ __forceinline__ RaySums spectral_sums(const Spec& S, float l1, float l2) {
+    const float a[1] = {l1}, b[1] = {l2};
+    RaySums s[1];
+    spectral_sums<NEED_S, COMP, 1>(S.e_hi - S.e_lo, a, b, s, [&](int e, float4& x, float2& y) {
+        const int i = S.e_lo + e;
+        x = make_float4(S.mu1l2[i], S.mu2l2[i], S.mu1[i], S.mu2[i]);
+        y = make_float2(S.i0l[i], S.i0h[i]);
+    });
+    return s[0];
 }
 
 }  // namespace deam

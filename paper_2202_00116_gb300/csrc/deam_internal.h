@@ -15,7 +15,8 @@ constexpr int kMaxE = 256;        // energy bins carried in the kernel-parameter
 constexpr int kTileK = 32;        // forward ray tile: channels (one warp) ...
 constexpr int kTileR = 4;         // ... x rows ...
 constexpr int kTileV = 2;         // ... x views
-constexpr int kFwdThreads = kTileK * kTileR * kTileV;  // rays per forward block (256)
+constexpr int kFwdThreads = kTileK * kTileR * kTileV;  // threads per forward block (256)
+constexpr int kRowsTV = kFwdThreads / 32;  // views of a forward block that projects several rows per thread
 
 // Geometry in voxel-index units, as read by both projector directions.  Every
 // per-ray quantity is derived from these tables by ray_inplane()/row terms with
@@ -23,6 +24,7 @@ constexpr int kFwdThreads = kTileK * kTileR * kTileV;  // rays per forward block
 // kernels compute bit-identical sample positions and weights.
 struct Geo {
     int nx, ny, nz, V, R, K;
+    int fwd_rows;            // rows a forward thread projects at once (forward_rows; host)
     float dx, dy;            // voxel edge lengths (mm)
     float dx_sdd, dy_sdd;    // dx / sdd, dy / sdd
     float dx_dy, dy_dx;      // dx / dy, dy / dx
@@ -249,7 +251,28 @@ cudaError_t launch_counter_inc(int* counter, cudaStream_t s);
 cudaError_t launch_inplane_table(const Geo& G, float4* ip4, float* ipL, cudaStream_t s);
 cudaError_t launch_layout(const float2* c, const float* m, int ones, float4* volX, float4* volY,
                           int nx, int ny, int nz, cudaStream_t s);
-int forward_blocks_per_sm();
+// Detector rows that a thread of the forward kernel projects at once (fwd_rows).
+//   1: one row, or a volume or cone too large for its floor and step tests
+//      (indices below 2^21, heights below 2048 slices).
+//   8: a volume at least twice as high as the detector covers at the axis: most
+//      rows meet it along the whole ray.  Against 4 rows, one launch: 11.5 / 12.9
+//      ms on a rotation of 512^2 x 64, 9.2 / 9.7 ms at 384^2 x 48, 3.1 / 3.3 ms on
+//      a rotation of 256^2 x 32 (against one row 15.4, 14.0 and 5.4 ms).
+//   4: thinner volumes, where rows in larger groups are carried along outside
+//      (256^2 x 16, 1440 views: 5.0 ms against 5.9 with 8 and 6.3 with 1), and
+//      detectors of few rows.
+inline int forward_rows(const deam_geometry& g) {
+    if (g.n_rows < 2 || g.nx >= (1 << 21) || g.ny >= (1 << 21) || g.nz >= 2048) return 1;
+    double w = 0.0;  // largest row height in slices
+    for (int r : {0, g.n_rows - 1}) {
+        const double h = (r - (g.n_rows - 1) / 2.0 + g.row_offset) * g.row_pitch / g.dz;
+        w = h > w ? h : -h > w ? -h : w;
+    }
+    if (!(w < 2048.0)) return 1;
+    return g.n_rows > 4 && g.nz * g.dz >= 2.0 * g.n_rows * g.row_pitch * g.sid / g.sdd ? 8 : 4;
+}
+// Blocks of the persistent forward grid: one resident wave, at most one per tile.
+int forward_blocks(const Geo& G, int sms);
 cudaError_t launch_forward(int mode, const Geo& G, const Spec& S, const FwdArgs& A, int n_blocks,
                            cudaStream_t s);
 cudaError_t launch_backward(int mode, const BwdPlan& P, const Geo& G, const BwdArgs& A, cudaStream_t s);

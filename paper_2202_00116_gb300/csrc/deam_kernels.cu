@@ -16,6 +16,7 @@
 
 #include "deam_epilogue.cuh"
 #include "deam_internal.h"
+#include "deam_pair.cuh"
 
 namespace deam {
 
@@ -35,15 +36,79 @@ __device__ __forceinline__ void clip_planes(float a, float b, float lo, float hi
     t1 = fminf(t1, fmaxf(u, w));
 }
 
+__host__ __device__ constexpr bool needs_spectrum(int mode) { return mode == FWD_LINE_G || mode == FWD_DEAM || mode == FWD_DEAM_F32; }
+
+// What becomes of ray (v, r, k) once its line integrals (l1, l2) and, where the
+// MODE has them, its spectral sums Q are known: the MODE's outputs.  rowf: the row
+// length factor.  Returns the ray's share of the block reduction (objective term,
+// l_1 for FWD_MAX; 0 otherwise).
+template <int MODE>
+__device__ __forceinline__ double ray_epilogue(const Geo& G, const FwdArgs& A, long long y, int k, float l1, float l2,
+                                               const RaySums& Q, float rowf) {
+    const long long nrays = (long long)G.V * G.R * G.K;
+    double out = 0.0;
+    // outputs are streamed (evict-first) so that they do not push the volume
+    // layouts out of L2
+    if (MODE == FWD_LINE) {
+        __stcs(&A.l_out[y], make_float2(l1, l2));
+    } else if (MODE == FWD_MASK) {
+        A.mask_out[y] = (uint8_t)(l1 >= A.threshold ? 3 : 0);  // one operator: both spectra
+    } else if (MODE == FWD_MAX) {
+        out = (double)l1;
+    } else if (MODE == FWD_LINE_G) {
+        const float bk = A.bowtie ? __ldg(&A.bowtie[k]) : 1.f;
+        if (A.l_out) __stcs(&A.l_out[y], make_float2(l1, l2));
+        __stcs(&A.g_out[y], Q.gl * bk);
+        __stcs(&A.g_out[nrays + y], Q.gh * bk);
+    } else {  // FWD_DEAM, FWD_DEAM_F32
+        const float bk = A.bowtie ? __ldg(&A.bowtie[k]) : 1.f;
+        const float gl = Q.gl * bk, gh = Q.gh * bk, s1l = Q.s1l * bk, s2l = Q.s2l * bk, s1h = Q.s1h * bk, s2h = Q.s2h * bk;
+        float4 P = make_float4(s1l + s1h, s2l + s2h, 0.f, 0.f);
+        // bit j of the mask: the ray is on the metal trace of spectrum j, where
+        // p = q (r_j = 1): no data term and no ratio contribution (Eq. 11)
+        const unsigned mk = A.mask != nullptr ? A.mask[y] : 0u;
+        float f = 0.f;
+        if (!(mk & 1u)) {
+            const float dl = __ldcs(&A.dt[y]);
+            if (gl > 0.f) {
+                const float u = (dl - gl) / gl;  // r_L - 1
+                P.z = fmaf(u, s1l, P.z);
+                P.w = fmaf(u, s2l, P.w);
+                f = fmaf(gl, idiv_phi(u), f);
+            } else if (dl > 0.f) {
+                f = INFINITY;
+            }
+        }
+        if (!(mk & 2u)) {
+            const float dh = __ldcs(&A.dt[nrays + y]);
+            if (gh > 0.f) {
+                const float u = (dh - gh) / gh;  // r_H - 1
+                P.z = fmaf(u, s1h, P.z);
+                P.w = fmaf(u, s2h, P.w);
+                f = fmaf(gh, idiv_phi(u), f);
+            } else if (dh > 0.f) {
+                f = INFINITY;
+            }
+        }
+        out = (double)f;
+        if (A.fold_rowfac) {  // the backprojector's internal form: h's row factor applied once per ray
+            P.x *= rowf;
+            P.y *= rowf;
+            P.z *= rowf;
+            P.w *= rowf;
+        }
+        __stcs(&A.payload[y], P);
+    }
+    return out;
+}
+
 // One ray (v, r, k): Joseph projection of both components, then the MODE's
 // epilogue.  Returns the ray's share of the block reduction (objective term,
 // l_1 for FWD_MAX, sample count for FWD_COUNT; 0 otherwise).
 template <int MODE>
 __device__ __forceinline__ double fwd_ray(const Geo& G, const Spec& S, const FwdArgs& A, int v, int r, int k) {
-    const long long nrays = (long long)G.V * G.R * G.K;
-    double out = 0.0;
     const long long y = ((long long)v * G.R + r) * G.K + k;
-    if (!DEAM_IN_BOUNDS(G, y >= 0 && y < nrays, SITE_FWD_RAY, y)) return out;
+    if (!DEAM_IN_BOUNDS(G, y >= 0 && y < (long long)G.V * G.R * G.K, SITE_FWD_RAY, y)) return 0.0;
     const float sz = __ldg(&G.view_z[v]);
     const float2 rw = make_float2(row_omega(G, r), __ldg(&G.row[r]).y);  // (omega_r, row length factor)
     const long long vk = (long long)v * G.K + k;
@@ -105,101 +170,256 @@ __device__ __forceinline__ double fwd_ray(const Geo& G, const Spec& S, const Fwd
         s1 += fmaf(wz, b1 - a1, a1);
         s2 += fmaf(wz, b2 - a2, a2);
     }
+    if (MODE == FWD_COUNT) return (double)nsamp;
     const float L = __fmul_rn(ip.Lxy, rw.y);
     const float l1 = s1 * L, l2 = s2 * L;
+    RaySums Q{};
+    if (needs_spectrum(MODE)) Q = spectral_sums<MODE != FWD_LINE_G, MODE != FWD_DEAM_F32>(S, l1, l2);
+    return ray_epilogue<MODE>(G, A, y, k, l1, l2, Q, rw.y);
+}
 
-    // outputs are streamed (evict-first) so that they do not push the volume
-    // layouts out of L2
-    if (MODE == FWD_LINE) {
-        __stcs(&A.l_out[y], make_float2(l1, l2));
-    } else if (MODE == FWD_MASK) {
-        A.mask_out[y] = (uint8_t)(l1 >= A.threshold ? 3 : 0);  // one operator: both spectra
-    } else if (MODE == FWD_MAX) {
-        out = (double)l1;
-    } else if (MODE == FWD_COUNT) {
-        out = (double)nsamp;
-    } else if (MODE == FWD_LINE_G) {
-        float gl, gh, a, b, c, d;
-        spectral_sums<false>(S, l1, l2, gl, gh, a, b, c, d);
-        const float bk = A.bowtie ? __ldg(&A.bowtie[k]) : 1.f;
-        if (A.l_out) __stcs(&A.l_out[y], make_float2(l1, l2));
-        __stcs(&A.g_out[y], gl * bk);
-        __stcs(&A.g_out[nrays + y], gh * bk);
-    } else {  // FWD_DEAM, FWD_DEAM_F32
-        float gl, gh, s1l, s2l, s1h, s2h;
-        spectral_sums<true, MODE == FWD_DEAM>(S, l1, l2, gl, gh, s1l, s2l, s1h, s2h);
-        const float bk = A.bowtie ? __ldg(&A.bowtie[k]) : 1.f;
-        gl *= bk; gh *= bk; s1l *= bk; s2l *= bk; s1h *= bk; s2h *= bk;
-        float4 P = make_float4(s1l + s1h, s2l + s2h, 0.f, 0.f);
-        // bit j of the mask: the ray is on the metal trace of spectrum j, where
-        // p = q (r_j = 1): no data term and no ratio contribution (Eq. 11)
-        const unsigned mk = A.mask != nullptr ? A.mask[y] : 0u;
-        float f = 0.f;
-        if (!(mk & 1u)) {
-            const float dl = __ldcs(&A.dt[y]);
-            if (gl > 0.f) {
-                const float u = (dl - gl) / gl;  // r_L - 1
-                P.z = fmaf(u, s1l, P.z);
-                P.w = fmaf(u, s2l, P.w);
-                f = fmaf(gl, idiv_phi(u), f);
-            } else if (dl > 0.f) {
-                f = INFINITY;
+struct VoxelPair {
+    pair32 a, b;  // voxels q and q + 1
+};
+// asks L2 to keep the line
+__device__ __forceinline__ VoxelPair load_pair(const float4* p, unsigned long long pol) {
+    VoxelPair v;
+    asm("ld.global.nc.L2::cache_hint.v2.u64 {%0, %1}, [%2], %3;" : "=l"(v.a), "=l"(v.b) : "l"(p), "l"(pol));
+    return v;
+}
+__device__ __forceinline__ pair32 lerp(pair32 a, pair32 b, pair32 w) { return fma2(w, sub2(b, a), a); }
+
+// Planes a .. b of RB rows' sums.  KIND 0: a row's sample lies in the slice pair of
+// the row below or in the next one; 1: anywhere; 2: anywhere, and perhaps outside
+// the volume.
+template <int KIND, int RB>
+__device__ __forceinline__ void fwd_planes(pair32 (&s)[RB], const float (&om)[RB], const InPlane& ip, float sz,
+                                           const float4* __restrict__ vol, unsigned long long pol, const Geo& G, int nq,
+                                           int first, int last) {
+    const int rs = nq + 1;           // pairs per (plane, z) row
+    const int ps = (G.nz + 2) * rs;  // pairs per plane
+    constexpr float kMagic = 12582912.f;  // 1.5 x 2^23: x + kMagic rounded down is floor(x) + kMagic (|x| < 2^22)
+    const float fnz = (float)G.nz;
+    const unsigned origin = 1u - 0x4B400000u - (0x4B400000u - 1u) * (unsigned)rs;  // takes the bits of q and z below to an index
+#pragma unroll 1
+    for (int p = first; p <= last; ++p) {
+        const float pf = (float)p;
+        const float fq = __fmaf_rn(pf, ip.bq, ip.aq);
+        const float t = ray_t(ip, pf);
+        const float mq = __fadd_rd(fq, kMagic);
+        const float wqs = fq - (mq - kMagic);
+        const pair32 wq = dup2(wqs);
+        const unsigned base = origin + (unsigned)(p * ps) + (unsigned)__float_as_int(mq);
+        float wz[RB];
+        int m[RB];  // bits of floor(fz) + kMagic: consecutive for consecutive slices
+        bool ok[RB];
+        VoxelPair h[RB], l[RB];
+#pragma unroll
+        for (int i = 0; i < RB; ++i) {
+            const float fz = row_fz(sz, om[i], t);
+            const float f = __fadd_rd(fz, kMagic);
+            wz[i] = fz - (f - kMagic);
+            m[i] = __float_as_int(f);
+            if (KIND == 2) {
+                ok[i] = fz >= -1.f && fz < fnz;
+                m[i] = min(max(m[i], 0x4B400000 - 1), 0x4B400000 - 1 + G.nz);
             }
         }
-        if (!(mk & 2u)) {
-            const float dh = __ldcs(&A.dt[nrays + y]);
-            if (gh > 0.f) {
-                const float u = (dh - gh) / gh;  // r_H - 1
-                P.z = fmaf(u, s1h, P.z);
-                P.w = fmaf(u, s2h, P.w);
-                f = fmaf(gh, idiv_phi(u), f);
-            } else if (dh > 0.f) {
-                f = INFINITY;
+#pragma unroll
+        for (int i = 0; i < RB; ++i) {
+            const unsigned e = base + (unsigned)m[i] * (unsigned)rs;
+            h[i] = l[i] = VoxelPair{};
+            if (!DEAM_IN_BOUNDS(G, (long long)e + rs < (long long)(ip.axis ? G.ny : G.nx) * ps, SITE_FWD_LAYOUT, e)) continue;
+            h[i] = load_pair(vol + e + rs, pol);
+            // the lower slice is the one above of the row below, or that row's own,
+            // unless the heights jump (else: one address for the whole warp)
+            if (i == 0) l[i] = load_pair(vol + e, pol);
+            else if (KIND > 0) l[i] = load_pair(vol + ((unsigned)(m[i] - m[i - 1]) > 1u ? e : 0u), pol);
+        }
+        pair32 lo, hi;
+#pragma unroll
+        for (int i = 0; i < RB; ++i) {
+            if (i == 0) {
+                lo = lerp(l[i].a, l[i].b, wq);
+            } else {
+                const unsigned d = m[i] - m[i - 1];
+                lo = d ? hi : lo;
+                if (KIND > 0) {
+                    const pair32 own = lerp(l[i].a, l[i].b, wq);
+                    lo = d > 1u ? own : lo;
+                }
             }
+            hi = lerp(h[i].a, h[i].b, wq);
+            const pair32 x = lerp(lo, hi, dup2(wz[i]));
+            if (KIND < 2 || ok[i]) s[i] = add2(s[i], x);
         }
-        out = (double)f;
-        if (A.fold_rowfac) {  // the backprojector's internal form: h's row factor applied once per ray
-            P.x *= rw.y;
-            P.y *= rw.y;
-            P.z *= rw.y;
-            P.w *= rw.y;
+    }
+}
+
+// RB rows r0 .. r0 + RB - 1 of (view v, channel k) at once: they cross the planes
+// at the same q and at rising heights, so the plane's terms are computed once, and
+// the lower slice of a row's sample is one that the row below has read and
+// interpolated along q (always so where a row rises by less than a slice).  The
+// values added are fwd_ray's, in its order: bit for bit the same sums.
+//
+// What bounds it: issue (fwd_ray sits at 0.5-0.6 per cycle and scheduler with its
+// L1 data path 65-87 % busy on two loads per sample).  Floors by the rounding of
+// an addition instead of the conversion unit, packed interpolation of the two
+// components, one to 1.25 loads per sample for half of the ray.  Spectral tables
+// in shared memory, read once for two rays (read from the constant bank per ray
+// the epilogue of 60 bins took 2.4 of 8.1 ms).  Predicated loads that skip a slice
+// already held cost more registers than they save requests (6.2 against 5.0 ms at
+// 256^2 x 16).
+template <int MODE, int RB>
+__device__ __forceinline__ double fwd_rows(const Geo& G, const FwdArgs& A, int v, int r0, int k, float2* sums,
+                                           const SpecTable& T, int bins) {
+    const float sz = __ldg(&G.view_z[v]);
+    const long long vk = (long long)v * G.K + k;
+    const InPlane ip = inplane_at(__ldg(&G.ip4[vk]), __ldg(&G.ipL[vk]));
+    const int nr = min(RB, G.R - r0);
+    const int np = ip.axis ? G.ny : G.nx;
+    const int nq = ip.axis ? G.nx : G.ny;
+    const float4* __restrict__ vol = ip.axis ? A.volY : A.volX;
+    unsigned long long pol;
+    asm("createpolicy.fractional.L2::evict_last.b64 %0, 1.0;" : "=l"(pol));
+    const float fnq = (float)nq, fnz = (float)G.nz;
+    float om[RB];  // a row past the last repeats it (and is not written)
+#pragma unroll
+    for (int i = 0; i < RB; ++i) om[i] = row_omega(G, r0 + min(i, nr - 1));
+    // planes whose sample lies in the volume: exactly along q; along z those at
+    // which the group's lowest row is below its top and the highest above its floor
+    float t0 = 0.f, t1 = (float)(np - 1);
+    clip_planes(ip.aq, ip.bq, -1.f, fnq, t0, t1);
+    const bool back = ip.tau0 + 0.5f * (t0 + t1) * ip.kappa < 0.f;
+    const float oa = back ? om[RB - 1] : om[0], ob = back ? om[0] : om[RB - 1];
+    clip_planes(fmaf(ip.tau0, oa, sz), ip.kappa * oa, -1e30f, fnz, t0, t1);
+    clip_planes(fmaf(ip.tau0, ob, sz), ip.kappa * ob, -1.f, 1e30f, t0, t1);
+    int p0 = 0, p1 = -1;
+    if (t0 <= t1) {
+        p0 = max(0, (int)floorf(t0) - 1);
+        p1 = min(np - 1, (int)ceilf(t1) + 1);
+    }
+    auto in_q = [&](int p) {
+        const float fq = __fmaf_rn((float)p, ip.bq, ip.aq);
+        return fq >= -1.f && fq < fnq;
+    };
+    while (p0 <= p1 && !in_q(p0)) ++p0;
+    while (p1 >= p0 && !in_q(p1)) --p1;
+    pair32 s[RB];
+#pragma unroll
+    for (int i = 0; i < RB; ++i) s[i] = pack2(0.f, 0.f);
+    // heights are monotone in p and in the row: all samples are inside the volume
+    // if the corner ones are
+    auto inside = [&](float o, int p) {
+        const float fz = row_fz(sz, o, ray_t(ip, (float)p));
+        return fz >= -1.f && fz < fnz;
+    };
+    if (p0 <= p1) {
+        if (inside(om[0], p0) && inside(om[0], p1) && inside(om[RB - 1], p0) && inside(om[RB - 1], p1)) {
+            // a row rises by t domega slices over the one below: by less than one up
+            // to t = 1 / domega (less 1e-3 for the rounding of heights below 2048)
+            const float tc = 0.999f / G.domega;
+            const bool up = ip.kappa > 0.f;  // (rows rise: t > 0)
+            const float pc = fminf(fmaxf(__fdividef(tc - ip.tau0, ip.kappa), -1.f), (float)np);
+            // planes [p0, pa) and [pa, p1] with the near ones first if t rises with p
+            int pa = up ? (int)floorf(pc) : (int)ceilf(pc) + 1;
+            pa = min(max(pa, p0), p1 + 1);
+#pragma unroll 1
+            for (int part = 0; part < 2; ++part) {
+                const int a = part ? pa : p0, b = part ? p1 : pa - 1;
+                if (up == (part == 0) && !back) fwd_planes<0, RB>(s, om, ip, sz, vol, pol, G, nq, a, b);
+                else fwd_planes<1, RB>(s, om, ip, sz, vol, pol, G, nq, a, b);
+            }
+        } else {
+            fwd_planes<2, RB>(s, om, ip, sz, vol, pol, G, nq, p0, p1);
         }
-        __stcs(&A.payload[y], P);
+    }
+    // the epilogue two rows at a time (one copy of its code, and one read of the
+    // spectral tables for both): the sums go through shared memory
+    static_assert(RB % 2 == 0, "rows are finished in pairs");
+#pragma unroll
+    for (int i = 0; i < RB; ++i) sums[i * kFwdThreads] = unpack2(s[i]);
+    double out = 0.0;
+#pragma unroll 1
+    for (int i = 0; i < RB; i += 2) {
+        float l1[2], l2[2], rowf[2];
+        RaySums Q[2];
+#pragma unroll
+        for (int j = 0; j < 2; ++j) {
+            rowf[j] = __ldg(&G.row[r0 + min(i + j, nr - 1)]).y;
+            const float L = __fmul_rn(ip.Lxy, rowf[j]);
+            const float2 q = sums[(i + j) * kFwdThreads];
+            l1[j] = q.x * L;
+            l2[j] = q.y * L;
+        }
+        if constexpr (needs_spectrum(MODE))
+            spectral_sums<MODE != FWD_LINE_G, MODE != FWD_DEAM_F32, 2>(bins, l1, l2, Q, [&](int e, float4& a, float2& b) {
+                a = T.a[e];
+                b = T.b[e];
+            });
+#pragma unroll
+        for (int j = 0; j < 2; ++j) {
+            const long long y = ((long long)v * G.R + r0 + i + j) * G.K + k;
+            if (i + j >= nr ||
+                !DEAM_IN_BOUNDS(G, y >= 0 && y < (long long)G.V * G.R * G.K, SITE_FWD_RAY, y))
+                continue;
+            const double o = ray_epilogue<MODE>(G, A, y, k, l1[j], l2[j], Q[j], rowf[j]);
+            if (MODE == FWD_DEAM_F32) out = (double)((float)out + (float)o);
+            else out = MODE == FWD_MAX ? fmax(out, o) : out + o;
+        }
     }
     return out;
 }
 
-// Ray tiles of 32 channels (one warp) x TR rows x TV views: the warps of a block
-// sample neighbouring rows and views in step, so they read largely the same
-// voxel pairs and share them in L1.
-template <int TR, int TV>
+// Ray tiles of 32 channels (one warp) x TR groups of RB rows x TV views: the warps
+// of a block sample neighbouring rows and views in step, so they read largely the
+// same voxel pairs and share them in L1.
+template <int TR, int TV, int RB>
 __device__ __forceinline__ bool ray_of_tile(const Geo& G, long long t, int& v, int& r, int& k) {
-    const int nkt = (G.K + 31) / 32, nrt = (G.R + TR - 1) / TR;
+    const int nkt = (G.K + 31) / 32, nrt = (G.R + TR * RB - 1) / (TR * RB);
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const int kt = (int)(t % nkt);
     const long long t2 = t / nkt;
     const int rt = (int)(t2 % nrt);
     const int vt = (int)(t2 / nrt);
     k = kt * 32 + lane;
-    r = rt * TR + (warp % TR);
+    r = (rt * TR + (warp % TR)) * RB;
     v = vt * TV + (warp / TR);
     return k < G.K && r < G.R && v < G.V;
 }
 
-template <int TR, int TV>
+template <int TR, int TV, int RB>
 __host__ __device__ __forceinline__ long long ray_tiles(const Geo& G) {
-    return (long long)((G.K + 31) / 32) * ((G.R + TR - 1) / TR) * ((G.V + TV - 1) / TV);
+    return (long long)((G.K + 31) / 32) * ((G.R + TR * RB - 1) / (TR * RB)) * ((G.V + TV - 1) / TV);
 }
 
-template <int MODE>
-__global__ void __launch_bounds__(kFwdThreads) fwd_kernel(const Geo G, const Spec S, const FwdArgs A) {
+// Tile of a block: one row per thread, or RB rows per thread and a view per warp
+// (two or four groups of rows per block, sharing fewer views, were 15-40 % slower).
+template <int RB>
+struct FwdTile {
+    static constexpr int R = RB > 1 ? 1 : kTileR, V = RB > 1 ? kRowsTV : kTileV;
+    // resident blocks per SM: 64, 80 and 128 registers a thread
+    static constexpr int kBlocks = RB > 4 ? 2 : RB > 1 ? 3 : 4;
+};
+
+template <int MODE, int RB>
+__global__ void __launch_bounds__(kFwdThreads, FwdTile<RB>::kBlocks) fwd_kernel(const Geo G, const Spec S, const FwdArgs A) {
+    constexpr int TR = FwdTile<RB>::R, TV = FwdTile<RB>::V;
+    __shared__ float2 sums[RB > 1 ? RB * kFwdThreads : 1];
+    __shared__ SpecTable table;
+    if constexpr (RB > 1 && needs_spectrum(MODE)) {
+        fill_table(table, S);
+        __syncthreads();
+    }
     double red = 0.0;  // FWD_DEAM: objective of this thread's rays; FWD_MAX: max l_1
     float redf = 0.f;  // FWD_DEAM_F32: the same in FP32
-    const long long ntiles = ray_tiles<kTileR, kTileV>(G);
+    const long long ntiles = ray_tiles<TR, TV, RB>(G);
     for (long long t = blockIdx.x; t < ntiles; t += gridDim.x) {
         int v, r, k;
-        if (!ray_of_tile<kTileR, kTileV>(G, t, v, r, k)) continue;
-        const double o = fwd_ray<MODE>(G, S, A, v, r, k);
+        if (!ray_of_tile<TR, TV, RB>(G, t, v, r, k)) continue;
+        double o;
+        if constexpr (RB > 1) o = fwd_rows<MODE, RB>(G, A, v, r, k, sums + threadIdx.x, table, S.e_hi - S.e_lo);
+        else o = fwd_ray<MODE>(G, S, A, v, r, k);
         if (MODE == FWD_DEAM_F32) redf += (float)o;
         else red = MODE == FWD_MAX ? fmax(red, o) : red + o;
     }
@@ -299,7 +519,7 @@ __global__ void __launch_bounds__(kFwdThreads, 5) fwd_batch_kernel(const BatchDe
         const int i = si;
         int v, r, k;
         double f = 0.0;
-        if (ray_of_tile<TR, TV>(sG, t - __ldg(&B.ftile_off[i]), v, r, k))
+        if (ray_of_tile<TR, TV, 1>(sG, t - __ldg(&B.ftile_off[i]), v, r, k))
             f = fwd_ray<FWD_DEAM>(sG, B.specs[i], sA, v, r, k);
         const double b = block_reduce<kFwdThreads, double>(f, false);
         if (threadIdx.x == 0) B.partial[t] = b;  // per tile: independent of the grid
@@ -536,33 +756,50 @@ cudaError_t launch_layout(const float2* c, const float* m, int ones, float4* vol
 // Resident blocks per SM of the heaviest single-scan forward kernel: the
 // persistent forward grid is this many blocks per SM (one wave; a larger grid
 // of equal-work blocks leaves a partial second wave).
-int forward_blocks_per_sm() {
+template <int RB>
+static long long resident_blocks(const Geo& G, int sms) {
     int a = 0, b = 0;
-    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&a, fwd_kernel<FWD_DEAM>, kFwdThreads, 0) != cudaSuccess ||
-        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&b, fwd_kernel<FWD_DEAM_F32>, kFwdThreads, 0) != cudaSuccess)
-        return 4;
-    return std::max(1, std::min(a, b));
+    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&a, fwd_kernel<FWD_DEAM, RB>, kFwdThreads, 0) != cudaSuccess ||
+        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&b, fwd_kernel<FWD_DEAM_F32, RB>, kFwdThreads, 0) != cudaSuccess)
+        a = b = FwdTile<RB>::kBlocks;
+    return std::min<long long>(ray_tiles<FwdTile<RB>::R, FwdTile<RB>::V, RB>(G), (long long)sms * std::max(1, std::min(a, b)));
 }
 
-cudaError_t launch_forward(int mode, const Geo& G, const Spec& S, const FwdArgs& A, int n_blocks, cudaStream_t s) {
+int forward_blocks(const Geo& G, int sms) {
+    return (int)(G.fwd_rows == 8   ? resident_blocks<8>(G, sms)
+                 : G.fwd_rows == 4 ? resident_blocks<4>(G, sms)
+                                   : resident_blocks<1>(G, sms));
+}
+
+template <int RB>
+static cudaError_t launch_fwd(int mode, const Geo& G, const Spec& S, const FwdArgs& A, int n_blocks, cudaStream_t s) {
     switch (mode) {
-        case FWD_LINE: fwd_kernel<FWD_LINE><<<n_blocks, kFwdThreads, 0, s>>>(G, S, A); break;
-        case FWD_LINE_G: fwd_kernel<FWD_LINE_G><<<n_blocks, kFwdThreads, 0, s>>>(G, S, A); break;
-        case FWD_DEAM: fwd_kernel<FWD_DEAM><<<n_blocks, kFwdThreads, 0, s>>>(G, S, A); break;
-        case FWD_MASK: fwd_kernel<FWD_MASK><<<n_blocks, kFwdThreads, 0, s>>>(G, S, A); break;
-        case FWD_MAX: fwd_kernel<FWD_MAX><<<n_blocks, kFwdThreads, 0, s>>>(G, S, A); break;
-        case FWD_COUNT: fwd_kernel<FWD_COUNT><<<n_blocks, kFwdThreads, 0, s>>>(G, S, A); break;
-        case FWD_DEAM_F32: fwd_kernel<FWD_DEAM_F32><<<n_blocks, kFwdThreads, 0, s>>>(G, S, A); break;
+        case FWD_LINE: fwd_kernel<FWD_LINE, RB><<<n_blocks, kFwdThreads, 0, s>>>(G, S, A); break;
+        case FWD_LINE_G: fwd_kernel<FWD_LINE_G, RB><<<n_blocks, kFwdThreads, 0, s>>>(G, S, A); break;
+        case FWD_DEAM: fwd_kernel<FWD_DEAM, RB><<<n_blocks, kFwdThreads, 0, s>>>(G, S, A); break;
+        case FWD_MASK: fwd_kernel<FWD_MASK, RB><<<n_blocks, kFwdThreads, 0, s>>>(G, S, A); break;
+        case FWD_MAX: fwd_kernel<FWD_MAX, RB><<<n_blocks, kFwdThreads, 0, s>>>(G, S, A); break;
+        case FWD_DEAM_F32: fwd_kernel<FWD_DEAM_F32, RB><<<n_blocks, kFwdThreads, 0, s>>>(G, S, A); break;
         default: return cudaErrorInvalidValue;
     }
     return cudaGetLastError();
 }
 
+cudaError_t launch_forward(int mode, const Geo& G, const Spec& S, const FwdArgs& A, int n_blocks, cudaStream_t s) {
+    if (mode == FWD_COUNT) {
+        fwd_kernel<FWD_COUNT, 1><<<n_blocks, kFwdThreads, 0, s>>>(G, S, A);
+        return cudaGetLastError();
+    }
+    return G.fwd_rows == 8   ? launch_fwd<8>(mode, G, S, A, n_blocks, s)
+           : G.fwd_rows == 4 ? launch_fwd<4>(mode, G, S, A, n_blocks, s)
+                             : launch_fwd<1>(mode, G, S, A, n_blocks, s);
+}
+
 long long forward_tiles(int shape, const Geo& G) {
     switch (shape) {
-        case 0: return ray_tiles<8, 1>(G);
-        case 1: return ray_tiles<4, 2>(G);
-        default: return ray_tiles<2, 4>(G);
+        case 0: return ray_tiles<8, 1, 1>(G);
+        case 1: return ray_tiles<4, 2, 1>(G);
+        default: return ray_tiles<2, 4, 1>(G);
     }
 }
 

@@ -134,8 +134,8 @@ __global__ void __launch_bounds__(kThreads) objective_image_kernel(const ScanGeo
         // data term is then left out (Eq. 11: p = q there)
         const unsigned mk = mask ? (unsigned)mask[y] : 0u;
         if ((mk & 3u) != 3u) {
-            float gl, gh, u1, u2, u3, u4;
-            deam::spectral_sums<false>(S, l1, l2, gl, gh, u1, u2, u3, u4);
+            const deam::RaySums q = deam::spectral_sums<false>(S, l1, l2);
+            float gl = q.gl, gh = q.gh;
             const float bk = BT.on ? BT.b[k] : 1.f;
             gl *= bk;
             gh *= bk;
