@@ -286,7 +286,6 @@ int deam_init(const deam_geometry* geom, const deam_spectra* spectra, const deam
                                              : 0.5 * std::min(g.dx, std::min(g.dy, g.nz > 1 ? g.dz : g.dx));
     int sms = 152;
     cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, ctx->device);
-    ctx->bwd = deam::bwd_plan(g.nx, g.ny, g.nz, deam::pick_slab(g.nz, g.n_rows, g.dz, g.row_pitch, g.sid, g.sdd), sms);
 
     // ---- geometry tables (double on the host, rounded once to float) ----
     const double X0 = g.cx - (g.nx - 1) / 2.0 * g.dx, Y0 = g.cy - (g.ny - 1) / 2.0 * g.dy,
@@ -309,8 +308,14 @@ int deam_init(const deam_geometry* geom, const deam_spectra* spectra, const deam
         const double w = (r - (g.n_rows - 1) / 2.0 + g.row_offset) * g.row_pitch;
         rw[r] = make_float2((float)(w / g.dz), (float)sqrt(1.0 + (w / g.sdd) * (w / g.sdd)));
     }
+    // rays in the plane of the slice: no source height, no row height
+    const bool flat = g.row_offset == 0.0 && std::all_of(vz.begin(), vz.end(), [](float z) { return z == 0.f; });
+    ctx->bwd = deam::bwd_plan(g, flat, sms);
     // per (slab, column tile) in the backprojector's block order
-    const std::vector<int2> sv = deam::tile_view_ranges(g, ctx->bwd.slab, deam::bwd_tile_x(ctx->bwd.vs), deam::bwd_tile_y(ctx->bwd.vs));
+    // (a single slice is seen by all views)
+    std::vector<int2> sv;
+    if (ctx->bwd.slab > 1)
+        sv = deam::tile_view_ranges(g, ctx->bwd.slab, deam::bwd_tile_x(ctx->bwd.vs), deam::bwd_tile_y(ctx->bwd.vs));
 
     Geo& G = ctx->G;
     G.nx = g.nx; G.ny = g.ny; G.nz = g.nz; G.V = g.n_views; G.R = g.n_rows; G.K = g.n_channels;

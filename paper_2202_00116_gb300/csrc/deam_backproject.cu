@@ -146,12 +146,77 @@ __device__ __forceinline__ CornerWindow corner_window(const Geo& G, int v, float
     return W;
 }
 
+// The 8 x 4 columns of a warp: a lane's place in the patch, and what eight views
+// ask of it (every lane looks at one view from one corner of the patch: done for
+// each column, a window costs as much as a row of samples).
+struct Patch {
+    int ix, iy;      // the lane's column
+    float wx, wy;    // its place between the corners (inside the image)
+    float cx, cy;    // the corner that the lane looks from
+    float u, hw;     // of the lane's view and corner; hw the largest of the corners
+    int row0, row1;  // rows of a pair of views (2 w, 2 w + 1) that can reach the slab
+
+    __device__ __forceinline__ Patch(const Geo& G, int x0, int y0, int lane) {
+        // lanes in 4 x 2 blocks of columns: the eight lanes of a 128-byte wavefront
+        // read few distinct channels whatever the view's direction
+        const int lx = (lane & 3) + ((lane >> 1) & 4), ly = ((lane >> 2) & 1) + ((lane >> 3) & 2);
+        ix = x0 + lx;
+        iy = y0 + ly;
+        const int ex = min(7, max(G.nx - 1 - x0, 0)), ey = min(3, max(G.ny - 1 - y0, 0));
+        wx = __fdividef((float)lx, (float)max(ex, 1));
+        wy = __fdividef((float)ly, (float)max(ey, 1));
+        cx = (float)(x0 + ((lane & 1) ? ex : 0));
+        cy = (float)(y0 + ((lane & 2) ? ey : 0));
+    }
+    // views vb .. vb + 7 (the last repeated beyond it): lane 4 w + c looks at view w
+    __device__ __forceinline__ void look(const Geo& G, int vb, int last, int lane, float zlo, float zhi) {
+        const CornerWindow C = corner_window(G, min(vb + (lane >> 2), last), cx, cy, zlo, zhi);
+        float lo = C.lo, hi = C.hi;
+        u = C.u;
+        hw = C.hw;
+#pragma unroll
+        for (int o = 1; o < 4; o <<= 1) {
+            hw = fmaxf(hw, __shfl_xor_sync(0xffffffffu, hw, o));
+            lo = fminf(lo, __shfl_xor_sync(0xffffffffu, lo, o));
+            hi = fmaxf(hi, __shfl_xor_sync(0xffffffffu, hi, o));
+        }
+        lo = fminf(lo, __shfl_xor_sync(0xffffffffu, lo, 4));  // both views of a pair
+        hi = fmaxf(hi, __shfl_xor_sync(0xffffffffu, hi, 4));
+        row0 = max(0, __float2int_ru(fminf(lo, (float)G.R)));
+        row1 = min(G.R - 1, __float2int_rd(fmaxf(fminf(hi, (float)G.R), -1.f)));
+    }
+    // channels [k0, k1] of view w whose rays can tap the lane's column
+    __device__ __forceinline__ void channels(const Geo& G, int w, int& k0, int& k1) const {
+        const float a = __shfl_sync(0xffffffffu, u, 4 * w), b = __shfl_sync(0xffffffffu, u, 4 * w + 1);
+        const float c = __shfl_sync(0xffffffffu, u, 4 * w + 2), d = __shfl_sync(0xffffffffu, u, 4 * w + 3);
+        const float h = __shfl_sync(0xffffffffu, hw, 4 * w);
+        const float lu = fmaf(wx, b - a, a), hu = fmaf(wx, d - c, c);
+        const float at = fmaf(wy, hu - lu, lu);
+        k0 = max(0, __float2int_ru(fmaxf(at - h, -1.f)));
+        k1 = min(G.K - 1, __float2int_rd(fminf(at + h, (float)G.K)));
+    }
+};
+
 // G neighbouring rays (v, k .. k + G - 1) at a column: Joseph length x in-plane
 // weight (0: the ray does not tap the column) and ray parameter.
 template <int G_>
 struct Rays {
     float c[G_], t[G_];
 };
+
+// One ray's c (0: it does not tap the column) and t, from its table entry vk
+__device__ __forceinline__ void tap_ray(const Geo& G, long long vk, float fix, float fiy, float& c, float& t) {
+    const InPlane ip = inplane_at(__ldg(&G.ip4[vk]), __ldg(&G.ipL[vk]));
+    const float pf = ip.axis ? fiy : fix, qf = ip.axis ? fix : fiy;
+    const float fq = __fmaf_rn(pf, ip.bq, ip.aq);
+    const float jq = floorf(fq);
+    const float aq = fq - jq;
+    float wq = 0.f;
+    if (jq == qf) wq = 1.f - aq;
+    else if (jq == qf - 1.f) wq = aq;
+    c = ip.Lxy * wq;
+    t = ray_t(ip, pf);
+}
 
 template <int G_>
 __device__ __forceinline__ void load_rays(const Geo& G, Rays<G_>& y, int v, int k, int k1, float fix, float fiy,
@@ -162,17 +227,8 @@ __device__ __forceinline__ void load_rays(const Geo& G, Rays<G_>& y, int v, int 
         y.c[g] = y.t[g] = 0.f;
         if (k + g <= k1 &&
             DEAM_IN_BOUNDS(G, k >= 0 && vk + g < (long long)G.V * G.K, SITE_BWD_TABLE, vk + g)) {
-            const InPlane ip = inplane_at(__ldg(&G.ip4[vk + g]), __ldg(&G.ipL[vk + g]));
-            const float pf = ip.axis ? fiy : fix, qf = ip.axis ? fix : fiy;
-            const float fq = __fmaf_rn(pf, ip.bq, ip.aq);
-            const float jq = floorf(fq);
-            const float aq = fq - jq;
-            float wq = 0.f;
-            if (jq == qf) wq = 1.f - aq;
-            else if (jq == qf - 1.f) wq = aq;
-            y.c[g] = ip.Lxy * wq;
-            y.t[g] = ray_t(ip, pf);
-            if (wq != 0.f) {
+            tap_ray(G, vk + g, fix, fiy, y.c[g], y.t[g]);
+            if (y.c[g] != 0.f) {
                 tmin = fminf(tmin, y.t[g]);
                 tmax = fmaxf(tmax, y.t[g]);
             }
@@ -198,6 +254,40 @@ __device__ __forceinline__ void add_sample(Sums<FOUR>& lo, Sums<FOUR>& hi, float
     add_scaled<FOUR>(hi, dup2(w1), P);
 }
 
+// A voxel's sums a = (b~_1, b~_2, delta_1, delta_2), or the two of A^T y or the
+// gradient, to their end: stored, or the c-step.  False: out of range (checked
+// builds).
+template <int MODE>
+__device__ __forceinline__ bool finish_voxel(const Geo& G, const BwdArgs& A, long long vi, float4 a,
+                                             unsigned long long& skipped) {
+    if (!DEAM_IN_BOUNDS(G, vi < (long long)G.nx * G.ny * G.nz, SITE_BWD_IMAGE, vi)) return false;
+    if (MODE != BWD_UPDATE) {  // A^T y, or the gradient delta_i
+        A.img[vi] = make_float2(a.x, a.y);
+        return true;
+    }
+    if (A.sums) {  // regularised c-step: reg_update_kernel finishes the update
+        A.sums[vi] = a;
+        return true;
+    }
+    float2 c = A.img[vi];
+    // c-step: c_i <- c_i - (1/Z) ln(b^_i / b~_i) = c_i - (1/Z) log1p(delta_i / b~_i);
+    // the ratio and its logarithm in FP64 (two per voxel and iteration)
+    if (a.x > 0.f && a.z > -a.x) {
+        c.x = (float)fma(-log1p((double)a.z / (double)a.x), A.invZ, (double)c.x);
+        if (A.clamp_nonneg) c.x = fmaxf(c.x, 0.f);
+    } else {
+        ++skipped;
+    }
+    if (a.y > 0.f && a.w > -a.y) {
+        c.y = (float)fma(-log1p((double)a.w / (double)a.y), A.invZ, (double)c.y);
+        if (A.clamp_nonneg) c.y = fmaxf(c.y, 0.f);
+    } else {
+        ++skipped;
+    }
+    A.img[vi] = c;
+    return true;
+}
+
 // One (column tile, z-slab) of the gather backprojection: the work of one block
 // of VS groups of TX x TY threads.  Each group takes every VS-th eight views;
 // their sums are added in a fixed order (deterministic).
@@ -213,11 +303,8 @@ __device__ __forceinline__ void bwd_tile(const Geo& G, const BwdArgs& A, Sums<MO
     // parameter, so their rows fall between the same slices at nearly the same turn
     const int tid = threadIdx.x % NT, group = threadIdx.x / NT;
     const int warp = tid >> 5, lane = tid & 31;
-    const int px0 = bx * TX + (warp % (TX / 8)) * 8, py0 = by * TY + (warp / (TX / 8)) * 4;  // the warp's patch
-    // lanes in 4 x 2 blocks of columns: the eight lanes of a 128-byte wavefront
-    // read few distinct channels whatever the view's direction
-    const int lx = (lane & 3) + ((lane >> 1) & 4), ly = ((lane >> 2) & 1) + ((lane >> 3) & 2);
-    const int ix = px0 + lx, iy = py0 + ly;
+    Patch patch(G, bx * TX + (warp % (TX / 8)) * 8, by * TY + (warp / (TX / 8)) * 4, lane);
+    const int ix = patch.ix, iy = patch.iy;
     const bool inside = ix < G.nx && iy < G.ny;
     const int z0 = slab * SLAB;
     constexpr int G_ = kRaysPerView;
@@ -229,49 +316,22 @@ __device__ __forceinline__ void bwd_tile(const Geo& G, const BwdArgs& A, Sums<MO
         __ldg(&A.slab_views[((long long)slab * ((G.ny + TY - 1) / TY) + by) * ((G.nx + TX - 1) / TX) + bx]);
     const float fix = (float)ix, fiy = (float)iy;
     const float zlo = (float)(z0 - 1), zhi = (float)(z0 + SLAB);
-    // the patch's corners (inside the image) and the lane's place between them
-    const int ex = min(7, max(G.nx - 1 - px0, 0)), ey = min(3, max(G.ny - 1 - py0, 0));
-    const float wx = __fdividef((float)lx, (float)max(ex, 1)), wy = __fdividef((float)ly, (float)max(ey, 1));
-    const float cx = (float)(px0 + ((lane & 1) ? ex : 0)), cy = (float)(py0 + ((lane & 2) ? ey : 0));
     for (int vb = vrange.x + 8 * group; vb <= vrange.y; vb += 8 * VS) {
-        // eight views at a time: every lane looks at one view from one corner of
-        // the warp's patch (a window costs as much as a row of samples)
-        const CornerWindow C = corner_window(G, min(vb + (lane >> 2), vrange.y), cx, cy, zlo, zhi);
-        float hw = C.hw, lo = C.lo, hi = C.hi;
-#pragma unroll
-        for (int o = 1; o < 4; o <<= 1) {
-            hw = fmaxf(hw, __shfl_xor_sync(0xffffffffu, hw, o));
-            lo = fminf(lo, __shfl_xor_sync(0xffffffffu, lo, o));
-            hi = fmaxf(hi, __shfl_xor_sync(0xffffffffu, hi, o));
-        }
-        lo = fminf(lo, __shfl_xor_sync(0xffffffffu, lo, 4));  // both views of a pair
-        hi = fmaxf(hi, __shfl_xor_sync(0xffffffffu, hi, 4));
-        const int row0 = max(0, __float2int_ru(fminf(lo, (float)G.R)));
-        const int row1 = min(G.R - 1, __float2int_rd(fmaxf(fminf(hi, (float)G.R), -1.f)));
+        patch.look(G, vb, vrange.y, lane, zlo, zhi);
         // Views in pairs: their samples of a row lie within a few hundredths of a
         // slice of each other, so nearly always all between the same two slices
         // (one read and write of their sums serves the rays of both)
         const int nv = min(8, vrange.y - vb + 1);
         for (int w = 0; w < nv; w += 2) {
             const int v = vb + w;
-            const int r0 = __shfl_sync(0xffffffffu, row0, 4 * w), r1 = __shfl_sync(0xffffffffu, row1, 4 * w);
-            float u[2], h[2];
-#pragma unroll
-            for (int q = 0; q < 2; ++q) {
-                const int l = 4 * (w + q);
-                const float a = __shfl_sync(0xffffffffu, C.u, l), b = __shfl_sync(0xffffffffu, C.u, l + 1);
-                const float c = __shfl_sync(0xffffffffu, C.u, l + 2), d = __shfl_sync(0xffffffffu, C.u, l + 3);
-                const float lu = fmaf(wx, b - a, a), hu = fmaf(wx, d - c, c);
-                u[q] = fmaf(wy, hu - lu, lu);
-                h[q] = __shfl_sync(0xffffffffu, hw, l);
-            }
+            const int r0 = __shfl_sync(0xffffffffu, patch.row0, 4 * w), r1 = __shfl_sync(0xffffffffu, patch.row1, 4 * w);
+            int ka0, ka1, kb0, kb1;
+            patch.channels(G, w, ka0, ka1);
+            patch.channels(G, w + 1, kb0, kb1);
             if (r0 > r1) continue;  // no row of these views reaches the slab
             if (!inside) continue;
             const bool second = w + 1 < nv;
-            const int ka0 = max(0, __float2int_ru(fmaxf(u[0] - h[0], -1.f)));
-            const int ka1 = min(G.K - 1, __float2int_rd(fminf(u[0] + h[0], (float)G.K)));
-            const int kb0 = max(0, __float2int_ru(fmaxf(u[1] - h[1], -1.f)));
-            const int kb1 = second ? min(G.K - 1, __float2int_rd(fminf(u[1] + h[1], (float)G.K))) : kb0 - 1;
+            if (!second) kb1 = kb0 - 1;
             const float sza = __ldg(&G.view_z[v]), szb = __ldg(&G.view_z[second ? v + 1 : v]);
             const int n = max(ka1 - ka0, kb1 - kb0);
             for (int j = 0; j <= n; j += G_) {
@@ -356,34 +416,88 @@ __device__ __forceinline__ void bwd_tile(const Geo& G, const BwdArgs& A, Sums<MO
             a.z = hi.x;
             a.w = hi.y;
         }
-        const long long vi = ((long long)iz * G.ny + iy) * G.nx + ix;
-        if (!DEAM_IN_BOUNDS(G, vi < (long long)G.nx * G.ny * G.nz, SITE_BWD_IMAGE, vi)) break;
-        if (!FOUR) {  // A^T y, or the gradient delta_i
-            A.img[vi] = make_float2(a.x, a.y);
-            continue;
-        }
-        if (A.sums) {  // regularised c-step: reg_update_kernel finishes the update
-            A.sums[vi] = a;
-            continue;
-        }
-        float2 c = A.img[vi];
-        // c-step: c_i <- c_i - (1/Z) ln(b^_i / b~_i) = c_i - (1/Z) log1p(delta_i / b~_i);
-        // the ratio and its logarithm in FP64 (two per voxel and iteration)
-        if (a.x > 0.f && a.z > -a.x) {
-            c.x = (float)fma(-log1p((double)a.z / (double)a.x), A.invZ, (double)c.x);
-            if (A.clamp_nonneg) c.x = fmaxf(c.x, 0.f);
-        } else {
-            ++skipped;
-        }
-        if (a.y > 0.f && a.w > -a.y) {
-            c.y = (float)fma(-log1p((double)a.w / (double)a.y), A.invZ, (double)c.y);
-            if (A.clamp_nonneg) c.y = fmaxf(c.y, 0.f);
-        } else {
-            ++skipped;
-        }
-        A.img[vi] = c;
+        if (!finish_voxel<MODE>(G, A, ((long long)iz * G.ny + iy) * G.nx + ix, a, skipped)) break;
     }
     if (FOUR && skipped) atomicAdd(A.skipped, skipped);
+}
+
+// One slice seen by one detector row (fan-beam scans): no rows and no slices to
+// walk, so a thread keeps its column's sums in registers.  A block is one 8 x 4
+// patch of columns; its VS warps take every VS-th eight views.  FLAT: the rays lie
+// in the slice (no cone, source at its height).
+template <int MODE, int VS, bool FLAT>
+__global__ void __launch_bounds__(32 * VS, 32 / VS) bwd_slice_kernel(const Geo G, const BwdArgs A) {
+    constexpr bool FOUR = MODE == BWD_UPDATE;
+    constexpr int G_ = kRaysPerView;
+    __shared__ Sums<FOUR> part[VS * 32];
+    const int lane = threadIdx.x & 31, group = threadIdx.x >> 5;
+    const int ntx = (G.nx + 7) / 8;
+    Patch patch(G, (blockIdx.x % ntx) * 8, (blockIdx.x / ntx) * 4, lane);
+    const bool inside = patch.ix < G.nx && patch.iy < G.ny;
+    const float fix = (float)patch.ix, fiy = (float)patch.iy;
+    Sums<FOUR> acc{};
+    for (int vb = 8 * group; vb < G.V; vb += 8 * VS) {
+        patch.look(G, vb, G.V - 1, lane, -1.f, 1.f);
+        const int nv = min(8, G.V - vb);
+        for (int w = 0; w < nv; ++w) {
+            int k0, k1;
+            patch.channels(G, w, k0, k1);
+            if (!inside) continue;
+            const int v = vb + w;
+            const long long vk = (long long)v * G.K;
+            const float sz = __ldg(&G.view_z[v]);
+            for (int k = k0; k <= k1; k += G_) {
+                float c[G_];
+                Sums<FOUR> P[G_];
+#pragma unroll
+                for (int g = 0; g < G_; ++g) {
+                    c[g] = 0.f;
+                    P[g] = Sums<FOUR>{};
+                    const long long i = vk + k + g;
+                    if (k + g > k1 || !DEAM_IN_BOUNDS(G, k >= 0 && i < (long long)G.V * G.K, SITE_BWD_TABLE, i)) continue;
+                    // read along with the table, whether the ray taps the column or not
+                    P[g] = ray_data<MODE>(A, i);
+                    float t;
+                    tap_ray(G, i, fix, fiy, c[g], t);
+                    if (!FLAT) {
+                        // the slice's share of a sample at height fz: 1 - |fz|
+                        const float fz = row_fz(sz, G.omega0, t);
+                        const float f = floorf(fz), w1 = c[g] * (fz - f);
+                        c[g] = f == 0.f ? c[g] - w1 : f == -1.f ? w1 : 0.f;
+                    }
+                }
+#pragma unroll
+                for (int g = 0; g < G_; ++g)
+                    if (c[g] != 0.f) add_scaled<FOUR>(acc, dup2(c[g]), P[g]);
+            }
+        }
+        __syncwarp();
+    }
+    part[threadIdx.x] = acc;
+    __syncthreads();
+    if (group != 0 || !inside) return;
+#pragma unroll
+    for (int g = 1; g < VS; ++g) add_to<FOUR>(acc, part[32 * g + lane]);
+    const float rowf = MODE == BWD_ADJOINT ? __ldg(&G.row[0]).y : 1.f;  // else the payload carries it
+    const float2 lo = unpack2(acc.a);
+    float4 a = make_float4(lo.x * rowf, lo.y * rowf, 0.f, 0.f);
+    if constexpr (FOUR) {
+        const float2 hi = unpack2(acc.b);
+        a.z = hi.x;
+        a.w = hi.y;
+    }
+    unsigned long long skipped = 0;
+    finish_voxel<MODE>(G, A, (long long)patch.iy * G.nx + patch.ix, a, skipped);
+    if (FOUR && skipped) atomicAdd(A.skipped, skipped);
+}
+
+template <int VS, bool FLAT>
+static cudaError_t launch_slice(int mode, const Geo& G, const BwdArgs& A, cudaStream_t s) {
+    const int blocks = ((G.nx + 7) / 8) * ((G.ny + 3) / 4);
+    if (mode == BWD_UPDATE) bwd_slice_kernel<BWD_UPDATE, VS, FLAT><<<blocks, 32 * VS, 0, s>>>(G, A);
+    else if (mode == BWD_GRADIENT) bwd_slice_kernel<BWD_GRADIENT, VS, FLAT><<<blocks, 32 * VS, 0, s>>>(G, A);
+    else bwd_slice_kernel<BWD_ADJOINT, VS, FLAT><<<blocks, 32 * VS, 0, s>>>(G, A);
+    return cudaGetLastError();
 }
 
 // Column tile of a block of VS view groups
@@ -439,6 +553,10 @@ static cudaError_t launch_bwd(int mode, const Geo& G, const BwdArgs& A, cudaStre
 cudaError_t launch_backward(int mode, const BwdPlan& P, const Geo& G, const BwdArgs& A, cudaStream_t s) {
 #define DEAM_BWD(SL, VS) \
     if (P.slab == SL && P.vs == VS) return launch_bwd<SL, VS>(mode, G, A, s);
+    if (P.slab == 1) {
+        if (P.flat) return P.vs == 4 ? launch_slice<4, true>(mode, G, A, s) : launch_slice<16, true>(mode, G, A, s);
+        return P.vs == 4 ? launch_slice<4, false>(mode, G, A, s) : launch_slice<16, false>(mode, G, A, s);
+    }
     DEAM_BWD(2, 4)
     DEAM_BWD(kMidSlab, 1)
     DEAM_BWD(kMidSlab, 2)

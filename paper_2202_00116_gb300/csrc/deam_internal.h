@@ -12,11 +12,7 @@
 namespace deam {
 
 constexpr int kMaxE = 256;        // energy bins carried in the kernel-parameter tables
-constexpr int kTileK = 32;        // forward ray tile: channels (one warp) ...
-constexpr int kTileR = 4;         // ... x rows ...
-constexpr int kTileV = 2;         // ... x views
-constexpr int kFwdThreads = kTileK * kTileR * kTileV;  // threads per forward block (256)
-constexpr int kRowsTV = kFwdThreads / 32;  // views of a forward block that projects several rows per thread
+constexpr int kFwdThreads = 256;  // threads per forward block
 
 // Geometry in voxel-index units, as read by both projector directions.  Every
 // per-ray quantity is derived from these tables by ray_inplane()/row terms with
@@ -224,15 +220,24 @@ inline int pick_slab(int nz, int n_rows, double dz, double row_pitch, double sid
 //   as fast as 2 and 3 % faster than 4.
 struct BwdPlan {
     int slab = 2, vs = 4;
+    bool flat = false;  // slab 1: all rays lie in the slice
 };
 constexpr int kMidSlab = 11, kDeepSlab = 16;
 constexpr int bwd_tile_x(int vs) { return vs == 1 ? 16 : 8; }
 constexpr int bwd_tile_y(int vs) { return vs == 4 ? 4 : 8; }
-inline BwdPlan bwd_plan(int nx, int ny, int nz, int slab_class, int sms) {
+inline BwdPlan bwd_plan(const deam_geometry& g, bool flat, int sms) {
     BwdPlan p;
+    const long long patches = (long long)((g.nx + 7) / 8) * ((g.ny + 3) / 4);
+    if (g.nz == 1 && g.n_rows == 1) {
+        p.slab = 1;
+        p.flat = flat;
+        p.vs = patches >= 16LL * sms ? 4 : 16;
+        return p;
+    }
+    const int slab_class = pick_slab(g.nz, g.n_rows, g.dz, g.row_pitch, g.sid, g.sdd);
     if (slab_class == 2) return p;
     p.slab = slab_class == 8 ? kMidSlab : kDeepSlab;
-    const long long warps = (long long)((nx + 7) / 8) * ((ny + 3) / 4) * ((nz + p.slab - 1) / p.slab);
+    const long long warps = patches * ((g.nz + p.slab - 1) / p.slab);
     const long long round = 20LL * sms;
     p.vs = warps >= 8 * round ? 1 : warps >= 4 * round ? 2 : 4;
     return p;

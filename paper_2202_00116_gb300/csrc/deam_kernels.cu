@@ -152,6 +152,26 @@ __device__ __forceinline__ double fwd_ray(const Geo& G, const Spec& S, const Fwd
     }
     // no per-sample test: the loop body is branch-free and unrolls, so the
     // loads of several planes are in flight at once
+    if (G.nz == 1 && sz == 0.f && rw.x == 0.f && nq < (1 << 21)) {
+        // a fan-beam ray in the plane of its one slice: all samples at height 0, so
+        // the slice above has no weight and is not read (one load and 9 instead of
+        // two and 22 instructions per sample)
+        const unsigned origin = 1u - 0x4B400000u + (unsigned)rs;  // takes the bits of q below to an index
+        constexpr float kMagic = 12582912.f;  // 1.5 x 2^23: x + kMagic rounded down is floor(x) + kMagic
+#pragma unroll 4
+        for (int p = p0; p <= p1; ++p) {
+            const float fq = __fmaf_rn((float)p, ip.bq, ip.aq);
+            const float m = __fadd_rd(fq, kMagic);
+            const float wq = fq - (m - kMagic);
+            const unsigned e = origin + (unsigned)(p * ps) + (unsigned)__float_as_int(m);
+            float4 lo = make_float4(0.f, 0.f, 0.f, 0.f);
+            if (DEAM_IN_BOUNDS(G, e < (unsigned)(np * ps), SITE_FWD_LAYOUT, e))
+                asm("ld.global.nc.L2::cache_hint.v4.f32 {%0,%1,%2,%3}, [%4], %5;" : "=f"(lo.x), "=f"(lo.y), "=f"(lo.z), "=f"(lo.w) : "l"(vol + e), "l"(pol));
+            s1 += fmaf(wq, lo.z - lo.x, lo.x);
+            s2 += fmaf(wq, lo.w - lo.y, lo.y);
+        }
+        p1 = p0 - 1;
+    }
 #pragma unroll 4
     for (int p = p0; p <= p1; ++p) {
         const float pf = (float)p;
@@ -393,18 +413,15 @@ __host__ __device__ __forceinline__ long long ray_tiles(const Geo& G) {
     return (long long)((G.K + 31) / 32) * ((G.R + TR * RB - 1) / (TR * RB)) * ((G.V + TV - 1) / TV);
 }
 
-// Tile of a block: one row per thread, or RB rows per thread and a view per warp
-// (two or four groups of rows per block, sharing fewer views, were 15-40 % slower).
-template <int RB>
-struct FwdTile {
-    static constexpr int R = RB > 1 ? 1 : kTileR, V = RB > 1 ? kRowsTV : kTileV;
-    // resident blocks per SM: 64, 80 and 128 registers a thread
-    static constexpr int kBlocks = RB > 4 ? 2 : RB > 1 ? 3 : 4;
-};
+// A block's warps take a view each (two or four groups of rows per block, sharing
+// fewer views, were 15-40 % slower at 8 rows per thread; at one row they leave
+// warps of a fan-beam scan without a ray).
+constexpr int kBlockViews = kFwdThreads / 32;
+// Resident blocks per SM: 64, 80 and 128 registers a thread at 1, 4 and 8 rows
+__host__ __device__ constexpr int fwd_min_blocks(int rb) { return rb > 4 ? 2 : rb > 1 ? 3 : 4; }
 
 template <int MODE, int RB>
-__global__ void __launch_bounds__(kFwdThreads, FwdTile<RB>::kBlocks) fwd_kernel(const Geo G, const Spec S, const FwdArgs A) {
-    constexpr int TR = FwdTile<RB>::R, TV = FwdTile<RB>::V;
+__global__ void __launch_bounds__(kFwdThreads, fwd_min_blocks(RB)) fwd_kernel(const Geo G, const Spec S, const FwdArgs A) {
     __shared__ float2 sums[RB > 1 ? RB * kFwdThreads : 1];
     __shared__ SpecTable table;
     if constexpr (RB > 1 && needs_spectrum(MODE)) {
@@ -413,10 +430,10 @@ __global__ void __launch_bounds__(kFwdThreads, FwdTile<RB>::kBlocks) fwd_kernel(
     }
     double red = 0.0;  // FWD_DEAM: objective of this thread's rays; FWD_MAX: max l_1
     float redf = 0.f;  // FWD_DEAM_F32: the same in FP32
-    const long long ntiles = ray_tiles<TR, TV, RB>(G);
+    const long long ntiles = ray_tiles<1, kBlockViews, RB>(G);
     for (long long t = blockIdx.x; t < ntiles; t += gridDim.x) {
         int v, r, k;
-        if (!ray_of_tile<TR, TV, RB>(G, t, v, r, k)) continue;
+        if (!ray_of_tile<1, kBlockViews, RB>(G, t, v, r, k)) continue;
         double o;
         if constexpr (RB > 1) o = fwd_rows<MODE, RB>(G, A, v, r, k, sums + threadIdx.x, table, S.e_hi - S.e_lo);
         else o = fwd_ray<MODE>(G, S, A, v, r, k);
@@ -761,8 +778,8 @@ static long long resident_blocks(const Geo& G, int sms) {
     int a = 0, b = 0;
     if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&a, fwd_kernel<FWD_DEAM, RB>, kFwdThreads, 0) != cudaSuccess ||
         cudaOccupancyMaxActiveBlocksPerMultiprocessor(&b, fwd_kernel<FWD_DEAM_F32, RB>, kFwdThreads, 0) != cudaSuccess)
-        a = b = FwdTile<RB>::kBlocks;
-    return std::min<long long>(ray_tiles<FwdTile<RB>::R, FwdTile<RB>::V, RB>(G), (long long)sms * std::max(1, std::min(a, b)));
+        a = b = fwd_min_blocks(RB);
+    return std::min<long long>(ray_tiles<1, kBlockViews, RB>(G), (long long)sms * std::max(1, std::min(a, b)));
 }
 
 int forward_blocks(const Geo& G, int sms) {

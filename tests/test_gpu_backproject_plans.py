@@ -36,9 +36,9 @@ def pkg():
 def _geo(**kw):
     """Helical geometry of the tests' scanner; fan and rows follow the sizes."""
     g = dict(nx=40, ny=36, nz=12, dx=4.0, dz=0.75, R=16, K=96, V=48, vpr=48, pitch=0.8, row_mm=0.75, start=0.3,
-             cx=0.0, cy=0.0, cz=0.0, dy=None, row_offset=0.0)
+             cx=0.0, cy=0.0, cz=0.0, dy=None, row_offset=0.0, feed=2.0)
     g.update(kw)
-    feed = g["pitch"] * g["R"] * g["row_mm"] if g["R"] > 1 else 2.0
+    feed = g["pitch"] * g["R"] * g["row_mm"] if g["R"] > 1 else g["feed"]
     fov = max(g["nx"] * g["dx"], g["ny"] * (g["dy"] or g["dx"]))
     return synth.Geometry(synth.HELICAL, g["nx"], g["ny"], g["nz"], g["dx"], g["dy"] or g["dx"], g["dz"], g["cx"],
                           g["cy"], g["cz"], 570.0, 1040.0, g["V"], g["vpr"], g["start"], feed,
@@ -50,6 +50,8 @@ def _geo(**kw):
 LARGE = {
     "two_groups": _geo(nx=390, ny=261, nz=41, dx=0.98, K=150, V=9, vpr=9, pitch=3.0),
     "one_group": _geo(nx=512, ny=509, nz=49, dx=0.98, K=200, V=7, vpr=7, pitch=3.0),
+    "slice_tilted_wide": _geo(nx=410, ny=397, nz=1, R=1, dx=0.9, K=150, V=11, vpr=11, feed=0.8),
+    "slice_wide": _geo(nx=410, ny=397, nz=1, R=1, dx=0.9, K=150, V=11, vpr=11, feed=0.0),
 }
 GEOMETRIES = {
     # split over four view groups: deep and shallow slab class, exact and ragged slices
@@ -66,6 +68,11 @@ GEOMETRIES = {
     "one_row": _geo(nz=9, R=1, V=64, vpr=64),
     "one_column": _geo(nx=1, ny=1, nz=9, dx=60.0, K=33),
     "huge_voxels": _geo(nx=8, ny=7, nz=5, dx=60.0, dz=2.0, K=64),
+    # one slice and one row: sixteen and four warps per patch, in the plane of the
+    # source and beside it
+    "slice": _geo(nx=45, ny=34, nz=1, R=1, K=90, V=70, vpr=70, feed=0.0),
+    "slice_few_views": _geo(nx=20, ny=19, nz=1, R=1, K=31, V=5, vpr=5, feed=0.0),
+    "slice_tilted": _geo(nx=45, ny=34, nz=1, R=1, K=90, V=70, vpr=70, feed=0.6, row_offset=0.3),
     "off_axis": _geo(nx=33, ny=38, dy=5.1, cx=9.0, cy=-6.0, cz=1.3, row_offset=0.35, R=5, nz=19),
 }
 
@@ -91,7 +98,8 @@ def test_adjoint_matches_oracle(pkg, name):
     gpu.close()
 
 
-@pytest.mark.parametrize("name", ["deep_ragged", "mid_ragged", "straddling", "two_slices", "one_row"])
+@pytest.mark.parametrize("name", ["deep_ragged", "mid_ragged", "straddling", "two_slices", "one_row", "slice",
+                                  "slice_tilted"])
 def test_sums_and_gradient_match_adjoint_of_payload(pkg, name):
     import oracle
     case = _case(GEOMETRIES[name])
