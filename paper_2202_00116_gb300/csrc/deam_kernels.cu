@@ -221,15 +221,19 @@ __device__ __forceinline__ void fwd_planes(pair32 (&s)[RB], const float (&om)[RB
     constexpr float kMagic = 12582912.f;  // 1.5 x 2^23: x + kMagic rounded down is floor(x) + kMagic (|x| < 2^22)
     const float fnz = (float)G.nz;
     const unsigned origin = 1u - 0x4B400000u - (0x4B400000u - 1u) * (unsigned)rs;  // takes the bits of q and z below to an index
+    const float4* __restrict__ above = vol + rs;
+    // the plane as running sums, and the slice above by its own pointer: no conversion,
+    // product or 64-bit addition per plane and load (384^2 x 48: 9.0 against 9.4 ms)
+    float pf = (float)first;
+    unsigned plane = origin + (unsigned)(first * ps);
 #pragma unroll 1
-    for (int p = first; p <= last; ++p) {
-        const float pf = (float)p;
+    for (int p = first; p <= last; ++p, pf += 1.f, plane += (unsigned)ps) {
         const float fq = __fmaf_rn(pf, ip.bq, ip.aq);
         const float t = ray_t(ip, pf);
         const float mq = __fadd_rd(fq, kMagic);
         const float wqs = fq - (mq - kMagic);
         const pair32 wq = dup2(wqs);
-        const unsigned base = origin + (unsigned)(p * ps) + (unsigned)__float_as_int(mq);
+        const unsigned base = plane + (unsigned)__float_as_int(mq);
         float wz[RB];
         int m[RB];  // bits of floor(fz) + kMagic: consecutive for consecutive slices
         bool ok[RB];
@@ -250,7 +254,7 @@ __device__ __forceinline__ void fwd_planes(pair32 (&s)[RB], const float (&om)[RB
             const unsigned e = base + (unsigned)m[i] * (unsigned)rs;
             h[i] = l[i] = VoxelPair{};
             if (!DEAM_IN_BOUNDS(G, (long long)e + rs < (long long)(ip.axis ? G.ny : G.nx) * ps, SITE_FWD_LAYOUT, e)) continue;
-            h[i] = load_pair(vol + e + rs, pol);
+            h[i] = load_pair(above + e, pol);
             // the lower slice is the one above of the row below, or that row's own,
             // unless the heights jump (else: one address for the whole warp)
             if (i == 0) l[i] = load_pair(vol + e, pol);
