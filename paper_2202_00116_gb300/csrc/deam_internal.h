@@ -141,7 +141,8 @@ struct FwdArgs {
     float2* l_out;        // FWD_LINE(_G): [V][R][K] line integrals (nullable in LINE_G)
     float* g_out;         // FWD_LINE_G: [2][V][R][K] expected counts
     const float* dt;      // FWD_DEAM: d~ [2][V][R][K]
-    const uint8_t* mask;  // FWD_DEAM: [V][R][K] metal traces, bit j = spectrum j (nullable: none)
+    const uint8_t* mask;  // FWD_DEAM: [V][R][K] metal traces, bit j = spectrum j (nullable: none);
+                          // FWD_LINE: project only the rays in or next to a trace (nullable: all)
     const float* bowtie;  // [K] (nullable: 1)
     float4* payload;      // FWD_DEAM: [V][R][K] (B~1, B~2, D1, D2)
     double* partial;      // FWD_DEAM: per-block objective; FWD_MAX: per-block max; FWD_COUNT: samples

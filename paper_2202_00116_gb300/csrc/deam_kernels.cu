@@ -421,6 +421,18 @@ __host__ __device__ __forceinline__ long long ray_tiles(const Geo& G) {
 // fewer views, were 15-40 % slower at 8 rows per thread; at one row they leave
 // warps of a fan-beam scan without a ray).
 constexpr int kBlockViews = kFwdThreads / 32;
+// Whether one of the rows r .. r + rows - 1 has a metal trace at channel k or next to
+// it.  Completing a sinogram reads the prior's line integrals in the trace and at
+// its ends only, so its projection takes these rays (a lane without one waits for
+// its warp, a warp without one goes on to the next tile).
+__device__ __forceinline__ bool near_trace(const Geo& G, const uint8_t* __restrict__ mask, int v, int r, int rows, int k) {
+    const uint8_t* __restrict__ m = mask + ((long long)v * G.R + r) * G.K;
+    const int kl = max(k - 1, 0), kr = min(k + 1, G.K - 1);
+    int any = 0;
+    for (int i = 0; i < min(rows, G.R - r); ++i, m += G.K) any |= __ldg(&m[kl]) | __ldg(&m[k]) | __ldg(&m[kr]);
+    return any != 0;
+}
+
 // Resident blocks per SM: 64, 80 and 128 registers a thread at 1, 4 and 8 rows
 __host__ __device__ constexpr int fwd_min_blocks(int rb) { return rb > 4 ? 2 : rb > 1 ? 3 : 4; }
 
@@ -438,6 +450,7 @@ __global__ void __launch_bounds__(kFwdThreads, fwd_min_blocks(RB)) fwd_kernel(co
     for (long long t = blockIdx.x; t < ntiles; t += gridDim.x) {
         int v, r, k;
         if (!ray_of_tile<1, kBlockViews, RB>(G, t, v, r, k)) continue;
+        if (MODE == FWD_LINE && A.mask && !near_trace(G, A.mask, v, r, RB, k)) continue;
         double o;
         if constexpr (RB > 1) o = fwd_rows<MODE, RB>(G, A, v, r, k, sums + threadIdx.x, table, S.e_hi - S.e_lo);
         else o = fwd_ray<MODE>(G, S, A, v, r, k);

@@ -644,17 +644,22 @@ int deam_mar_init(deam_ctx* ctx, const deam_mar_params* P, const float* prior_in
             CK(cudaGetLastError());
         }
         // the prior's projection: Joseph forward projection of (prior, 0) into
-        // l (float2 per ray; NMAR reads its first component)
-        int rc = deam::build_layouts(ctx, nullptr, prior, 0, s);
-        if (rc != DEAM_OK) return rc;
-        deam::FwdArgs A = deam::fwd_args(ctx);
-        A.l_out = l;
-        CK(deam::launch_forward(deam::FWD_LINE, ctx->G, ctx->S, A, ctx->n_fwd_blocks, s));
+        // l (float2 per ray; NMAR reads its first component).  Only the rays in or
+        // next to a trace are projected, the others stay unset and have no use
+        // (256^2 x 32, 37.4 M rays, two rods: 7.2 ms for all of them, 1.7 for these)
+        if (ctx->mask_set) {
+            const int rc = deam::build_layouts(ctx, nullptr, prior, 0, s);
+            if (rc != DEAM_OK) return rc;
+            deam::FwdArgs A = deam::fwd_args(ctx);
+            A.l_out = l;
+            A.mask = ctx->mask;
+            CK(deam::launch_forward(deam::FWD_LINE, ctx->G, ctx->S, A, ctx->n_fwd_blocks, s));
+        }
         for (int j = 0; j < 2; ++j) {
-            rc = complete(ctx, p + (size_t)j * nr, (const float*)l, 2, j, (float)P->eps, t + (size_t)j * nr, s);
+            const int rc = complete(ctx, p + (size_t)j * nr, (const float*)l, 2, j, (float)P->eps, t + (size_t)j * nr, s);
             if (rc != DEAM_OK) return rc;
         }
-        rc = fbp(ctx, t, 2, p, mu, s);  // both spectra (the sinograms p are done with)
+        const int rc = fbp(ctx, t, 2, p, mu, s);  // both spectra (the sinograms p are done with)
         if (rc != DEAM_OK) return rc;
         const double ia = P->calib[3] / det, ib = -P->calib[1] / det, ic = -P->calib[2] / det, id = P->calib[0] / det;
         decompose_kernel<<<grid_for(nv, 256), 256, 0, s>>>(mu, nv, (float)ia, (float)ib, (float)ic, (float)id,
