@@ -31,12 +31,13 @@ namespace deam {
 // 512^2 x 64 scan, 20.5 -> 8.6 ms on one of the 256^2 x 32 scan.  Measured and
 // slower: sums in registers with the slices unrolled (37.5 ms on the first),
 // four views per turn (29-50 ms), first moments of the rays' heights instead of
-// each ray's own weights (faster by 5 % but no longer the forward's weights).
+// each ray's own weights (32.6 ms, and no longer the forward's weights).
 constexpr int kBwdThreads = 128;
 // Rays of a view that one turn of the row loop takes (more rays: more turns).
 // Four at 5 blocks of 128 threads per SM; three at 6 blocks are as fast at 2.6
 // rays per view and 8 % slower at 3.5 (384^2 x 48 on 816 channels).
 constexpr int kRaysPerView = 4;
+
 
 // A ray's data, or the sums of a voxel: (b~_1, b~_2) and, for the c-step, also
 // (delta_1, delta_2).  The gradient carries the second pair alone, the plain
@@ -97,7 +98,9 @@ struct CornerWindow {
     float u, hw, lo, hi;
 };
 
+template <int C>
 __device__ __forceinline__ CornerWindow corner_window(const Geo& G, int v, float fix, float fiy, float zlo, float zhi) {
+    constexpr float kDiag = 64.f * C * C + 32.f * (C - 1);  // over the patch's diagonal, squared
     CornerWindow W;
     const float4 vw = __ldg(&G.view4[v]);
     const float sz = __ldg(&G.view_z[v]);
@@ -120,7 +123,7 @@ __device__ __forceinline__ CornerWindow corner_window(const Geo& G, int v, float
     // channels.)
     const float edge = fmaxf(fabsf(px) * G.dy, fabsf(py) * G.dx) * inv * 1.001f;
     const float bend = rho * rho;
-    W.hw = fmaf(fmaf(edge * rest, fmaf(64.f, bend, 1.f), 8.f * bend), G.inv_dgamma, 0.05f);
+    W.hw = fmaf(fmaf(edge * rest, fmaf(kDiag, bend, 1.f), 0.125f * kDiag * bend), G.inv_dgamma, 0.05f);
     W.u = fmaf(fan_angle(crs, dot), G.inv_dgamma, G.chan_c0);
     W.lo = 0.f;
     W.hi = (float)(G.R - 1);
@@ -137,7 +140,7 @@ __device__ __forceinline__ CornerWindow corner_window(const Geo& G, int v, float
         W.lo = ulo - off - fmaf(fabsf(ulo), share, 0.02f);
         W.hi = uhi - off + fmaf(fabsf(uhi), share, 0.02f);
     }
-    if (rho > 0.1f) {  // voxels too large for these bounds: every channel and row
+    if (rho * C > 0.1f) {  // voxels too large for these bounds: every channel and row
         W.u = 0.f;
         W.hw = 1e9f;
         W.lo = 0.f;
@@ -149,51 +152,65 @@ __device__ __forceinline__ CornerWindow corner_window(const Geo& G, int v, float
 // The 8 x 4 columns of a warp: a lane's place in the patch, and what eight views
 // ask of it (every lane looks at one view from one corner of the patch: done for
 // each column, a window costs as much as a row of samples).
+template <int C>
 struct Patch {
-    int ix, iy;      // the lane's column
-    float wx, wy;    // its place between the corners (inside the image)
-    float cx, cy;    // the corner that the lane looks from
-    float u, hw;     // of the lane's view and corner; hw the largest of the corners
-    int row0, row1;  // rows of a pair of views (2 w, 2 w + 1) that can reach the slab
+    int ix, iy;       // the lane's first column
+    float mx, my;     // its columns' centre in patch widths from the patch's (inside the image)
+    float rx, ry;     // 1 / patch widths
+    float cx, cy;     // the corner that the lane looks from
+    float u, ux, uy;  // of the lane's view: channel coordinate at the patch's centre, and its change over the patch
+    float hw;         // half width of the window of the columns of any lane
+    int row0, row1;   // rows of a pair of views (2 w, 2 w + 1) that can reach the slab
 
     __device__ __forceinline__ Patch(const Geo& G, int x0, int y0, int lane) {
         // lanes in 4 x 2 blocks of columns: the eight lanes of a 128-byte wavefront
         // read few distinct channels whatever the view's direction
         const int lx = (lane & 3) + ((lane >> 1) & 4), ly = ((lane >> 2) & 1) + ((lane >> 3) & 2);
-        ix = x0 + lx;
-        iy = y0 + ly;
-        const int ex = min(7, max(G.nx - 1 - x0, 0)), ey = min(3, max(G.ny - 1 - y0, 0));
-        wx = __fdividef((float)lx, (float)max(ex, 1));
-        wy = __fdividef((float)ly, (float)max(ey, 1));
+        ix = x0 + C * lx;
+        iy = y0 + C * ly;
+        const int ex = min(8 * C - 1, max(G.nx - 1 - x0, 0)), ey = min(4 * C - 1, max(G.ny - 1 - y0, 0));
+        constexpr float kHalf = 0.5f * (C - 1);
+        rx = __fdividef(1.f, (float)max(ex, 1));
+        ry = __fdividef(1.f, (float)max(ey, 1));
+        mx = ((float)(C * lx) + kHalf) * rx - 0.5f;
+        my = ((float)(C * ly) + kHalf) * ry - 0.5f;
         cx = (float)(x0 + ((lane & 1) ? ex : 0));
         cy = (float)(y0 + ((lane & 2) ? ey : 0));
     }
     // views vb .. vb + 7 (the last repeated beyond it): lane 4 w + c looks at view w
     __device__ __forceinline__ void look(const Geo& G, int vb, int last, int lane, float zlo, float zhi) {
-        const CornerWindow C = corner_window(G, min(vb + (lane >> 2), last), cx, cy, zlo, zhi);
-        float lo = C.lo, hi = C.hi;
-        u = C.u;
-        hw = C.hw;
+        const CornerWindow win = corner_window<C>(G, min(vb + (lane >> 2), last), cx, cy, zlo, zhi);
+        float lo = win.lo, hi = win.hi;
+        hw = win.hw;
 #pragma unroll
         for (int o = 1; o < 4; o <<= 1) {
             hw = fmaxf(hw, __shfl_xor_sync(0xffffffffu, hw, o));
             lo = fminf(lo, __shfl_xor_sync(0xffffffffu, lo, o));
             hi = fmaxf(hi, __shfl_xor_sync(0xffffffffu, hi, o));
         }
+        // the plane through the corners' coordinates; what they are off it by, and
+        // (several columns per lane) the way from the centre to any of them, widen
+        // the window
+        const float a = __shfl_sync(0xffffffffu, win.u, lane & ~3), b = __shfl_sync(0xffffffffu, win.u, lane & ~3 | 1);
+        const float c = __shfl_sync(0xffffffffu, win.u, lane & ~3 | 2), d = __shfl_sync(0xffffffffu, win.u, lane | 3);
+        u = 0.25f * ((a + b) + (c + d));
+        ux = 0.5f * ((b - a) + (d - c));
+        uy = 0.5f * ((c - a) + (d - b));
+        hw += 0.25f * fabsf((b - a) - (d - c));
+        if (C > 1) hw += 0.5f * (C - 1) * (fabsf(ux) * rx + fabsf(uy) * ry);
         lo = fminf(lo, __shfl_xor_sync(0xffffffffu, lo, 4));  // both views of a pair
         hi = fmaxf(hi, __shfl_xor_sync(0xffffffffu, hi, 4));
         row0 = max(0, __float2int_ru(fminf(lo, (float)G.R)));
         row1 = min(G.R - 1, __float2int_rd(fmaxf(fminf(hi, (float)G.R), -1.f)));
     }
-    // channels [k0, k1] of view w whose rays can tap the lane's column
+    // channels [k0, k1] of view w whose rays can tap the lane's columns
     __device__ __forceinline__ void channels(const Geo& G, int w, int& k0, int& k1) const {
-        const float a = __shfl_sync(0xffffffffu, u, 4 * w), b = __shfl_sync(0xffffffffu, u, 4 * w + 1);
-        const float c = __shfl_sync(0xffffffffu, u, 4 * w + 2), d = __shfl_sync(0xffffffffu, u, 4 * w + 3);
         const float h = __shfl_sync(0xffffffffu, hw, 4 * w);
-        const float lu = fmaf(wx, b - a, a), hu = fmaf(wx, d - c, c);
-        const float at = fmaf(wy, hu - lu, lu);
-        k0 = max(0, __float2int_ru(fmaxf(at - h, -1.f)));
-        k1 = min(G.K - 1, __float2int_rd(fminf(at + h, (float)G.K)));
+        float at = __shfl_sync(0xffffffffu, u, 4 * w);
+        at = fmaf(mx, __shfl_sync(0xffffffffu, ux, 4 * w), at);
+        at = fmaf(my, __shfl_sync(0xffffffffu, uy, 4 * w), at);
+        k0 = __float2int_ru(fmaxf(at - h, 0.f));
+        k1 = __float2int_rd(fminf(at + h, (float)(G.K - 1)));
     }
 };
 
@@ -303,7 +320,7 @@ __device__ __forceinline__ void bwd_tile(const Geo& G, const BwdArgs& A, Sums<MO
     // parameter, so their rows fall between the same slices at nearly the same turn
     const int tid = threadIdx.x % NT, group = threadIdx.x / NT;
     const int warp = tid >> 5, lane = tid & 31;
-    Patch patch(G, bx * TX + (warp % (TX / 8)) * 8, by * TY + (warp / (TX / 8)) * 4, lane);
+    Patch<1> patch(G, bx * TX + (warp % (TX / 8)) * 8, by * TY + (warp / (TX / 8)) * 4, lane);
     const int ix = patch.ix, iy = patch.iy;
     const bool inside = ix < G.nx && iy < G.ny;
     const int z0 = slab * SLAB;
@@ -421,82 +438,142 @@ __device__ __forceinline__ void bwd_tile(const Geo& G, const BwdArgs& A, Sums<MO
     if (FOUR && skipped) atomicAdd(A.skipped, skipped);
 }
 
-// One slice seen by one detector row (fan-beam scans): no rows and no slices to
-// walk, so a thread keeps its column's sums in registers.  A block is one 8 x 4
-// patch of columns; its VS warps take every VS-th eight views.  FLAT: the rays lie
-// in the slice (no cone, source at its height).
-template <int MODE, int VS, bool FLAT>
-__global__ void __launch_bounds__(32 * VS, 32 / VS) bwd_slice_kernel(const Geo G, const BwdArgs A) {
+// The sums of a thread's C x C columns (0, 0), (1, 0), (0, 1), (1, 1) over every
+// VS-th eight views.  EXACT leaves out the rays whose weight is zero, else they are
+// added with it.
+template <int MODE, int C, int VS, bool FLAT, bool EXACT>
+__device__ __forceinline__ void slice_sums(const Geo& G, const BwdArgs& A, Patch<C>& patch, bool inside, int group,
+                                           int lane, Sums<MODE == BWD_UPDATE> (&acc)[C * C]) {
     constexpr bool FOUR = MODE == BWD_UPDATE;
-    constexpr int G_ = kRaysPerView;
-    __shared__ Sums<FOUR> part[VS * 32];
-    const int lane = threadIdx.x & 31, group = threadIdx.x >> 5;
-    const int ntx = (G.nx + 7) / 8;
-    Patch patch(G, (blockIdx.x % ntx) * 8, (blockIdx.x / ntx) * 4, lane);
-    const bool inside = patch.ix < G.nx && patch.iy < G.ny;
+    constexpr int NV = C > 1 ? 1 : 4;  // views abreast, a ray of each per turn
     const float fix = (float)patch.ix, fiy = (float)patch.iy;
-    Sums<FOUR> acc{};
+#pragma unroll
+    for (int j = 0; j < C * C; ++j) acc[j] = Sums<FOUR>{};
     for (int vb = 8 * group; vb < G.V; vb += 8 * VS) {
         patch.look(G, vb, G.V - 1, lane, -1.f, 1.f);
         const int nv = min(8, G.V - vb);
-        for (int w = 0; w < nv; ++w) {
-            int k0, k1;
-            patch.channels(G, w, k0, k1);
+        for (int w = 0; w < nv; w += NV) {
+            int k0[NV], k1[NV], n = -1;
+#pragma unroll
+            for (int u = 0; u < NV; ++u) {
+                patch.channels(G, w + u, k0[u], k1[u]);
+                if (NV > 1 && w + u >= nv) k1[u] = k0[u] - 1;
+                n = max(n, k1[u] - k0[u]);
+            }
             if (!inside) continue;
             const int v = vb + w;
-            const long long vk = (long long)v * G.K;
-            const float sz = __ldg(&G.view_z[v]);
-            for (int k = k0; k <= k1; k += G_) {
-                float c[G_];
-                Sums<FOUR> P[G_];
+#pragma unroll 1
+            for (int j = 0; j <= n; ++j) {
+                InPlane ip[NV];
+                Sums<FOUR> P[NV];
+                float sz[NV];
 #pragma unroll
-                for (int g = 0; g < G_; ++g) {
-                    c[g] = 0.f;
+                for (int g = 0; g < NV; ++g) {
+                    const int k = k0[g] + j;
+                    const bool on = NV == 1 || k <= k1[g];
+                    const long long i = on ? (long long)(v + g) * G.K + k : 0;
+                    ip[g] = InPlane{};
                     P[g] = Sums<FOUR>{};
-                    const long long i = vk + k + g;
-                    if (k + g > k1 || !DEAM_IN_BOUNDS(G, k >= 0 && i < (long long)G.V * G.K, SITE_BWD_TABLE, i)) continue;
-                    // read along with the table, whether the ray taps the column or not
+                    sz[g] = __ldg(&G.view_z[on ? v + g : 0]);
+                    if (!DEAM_IN_BOUNDS(G, i >= 0 && i < (long long)G.V * G.K, SITE_BWD_TABLE, i)) continue;
                     P[g] = ray_data<MODE>(A, i);
-                    float t;
-                    tap_ray(G, i, fix, fiy, c[g], t);
-                    if (!FLAT) {
-                        // the slice's share of a sample at height fz: 1 - |fz|
-                        const float fz = row_fz(sz, G.omega0, t);
-                        const float f = floorf(fz), w1 = c[g] * (fz - f);
-                        c[g] = f == 0.f ? c[g] - w1 : f == -1.f ? w1 : 0.f;
-                    }
+                    ip[g] = inplane_at(__ldg(&G.ip4[i]), __ldg(&G.ipL[i]));
+                    if (!on) ip[g].Lxy = 0.f;
                 }
 #pragma unroll
-                for (int g = 0; g < G_; ++g)
-                    if (c[g] != 0.f) add_scaled<FOUR>(acc, dup2(c[g]), P[g]);
+                for (int g = 0; g < NV; ++g) {
+                    // planes p0 .. p0 + C - 1, at each of them the shares of q0 .. q0 + C - 1
+                    const float p0 = ip[g].axis ? fiy : fix, q0 = ip[g].axis ? fix : fiy;
+                    float c[C][C];
+#pragma unroll
+                    for (int p = 0; p < C; ++p) {
+                        const float pf = p0 + (float)p;
+                        const float d = __fmaf_rn(pf, ip[g].bq, ip[g].aq) - q0;
+                        float L = ip[g].Lxy;
+                        if (!FLAT) L *= __saturatef(1.f - fabsf(row_fz(sz[g], G.omega0, ray_t(ip[g], pf))));
+#pragma unroll
+                        for (int q = 0; q < C; ++q) c[p][q] = L * __saturatef(1.f - fabsf(d - (float)q));
+                    }
+#pragma unroll
+                    for (int j = 0; j < C * C; ++j) {
+                        const float x = ip[g].axis ? c[j / C][j % C] : c[j % C][j / C];
+                        if (!EXACT || x != 0.f) add_scaled<FOUR>(acc[j], dup2(x), P[g]);
+                    }
+                }
             }
         }
         __syncwarp();
     }
-    part[threadIdx.x] = acc;
-    __syncthreads();
-    if (group != 0 || !inside) return;
+}
+
+// One slice seen by one detector row (fan-beam scans): no rows and no slices to
+// walk, so a thread keeps the sums of its C x C columns in registers.  A block is one
+// 8 C x 4 C patch of columns; its VS warps take every VS-th eight views.  FLAT: the
+// rays lie in the slice (no cone, source at its height).
+//
+// What bounds it: issue (0.85 per cycle and scheduler).  2 x 2 columns share the
+// window, the ray's table entry and its data, and a plane's position gives two
+// weights: 5.5 rays instead of four times 3.5, 80 instead of 165 instructions per
+// column and view, 1.61 -> 0.87 ms at 512^2 x 1160 views with one ray per turn (two,
+// three, four: 0.91, 0.98, 1.18 ms).  Small images leave too few patches for that:
+// one column per thread, and the rays of four views in flight per turn to cover the
+// loads (128^2 x 360 views: 53 us; 58 with four rays of one view, 57 with 2 x 2
+// columns).  Skipping the columns that a ray does not tap, instead of adding zeros
+// and looking for infinities afterwards, was 1.15 against 0.98 ms.
+template <int MODE, int C, int VS, bool FLAT>
+__global__ void __launch_bounds__(32 * VS, 32 / VS) bwd_slice_kernel(const Geo G, const BwdArgs A) {
+    constexpr bool FOUR = MODE == BWD_UPDATE;
+    __shared__ Sums<FOUR> part[VS * 32];
+    const int lane = threadIdx.x & 31, group = threadIdx.x >> 5;
+    const int ntx = (G.nx + 8 * C - 1) / (8 * C);
+    Patch<C> patch(G, (blockIdx.x % ntx) * 8 * C, (blockIdx.x / ntx) * 4 * C, lane);
+    const bool inside = patch.ix < G.nx && patch.iy < G.ny;
+    Sums<FOUR> acc[C * C];
+    slice_sums<MODE, C, VS, FLAT, false>(G, A, patch, inside, group, lane, acc);
+    // a weight of zero takes nothing from finite data; where a sum has met an
+    // infinity or a NaN, the rays that tap the column decide
+    float zero = 0.f;
 #pragma unroll
-    for (int g = 1; g < VS; ++g) add_to<FOUR>(acc, part[32 * g + lane]);
-    const float rowf = MODE == BWD_ADJOINT ? __ldg(&G.row[0]).y : 1.f;  // else the payload carries it
-    const float2 lo = unpack2(acc.a);
-    float4 a = make_float4(lo.x * rowf, lo.y * rowf, 0.f, 0.f);
-    if constexpr (FOUR) {
-        const float2 hi = unpack2(acc.b);
-        a.z = hi.x;
-        a.w = hi.y;
+    for (int j = 0; j < C * C; ++j) {
+        const float2 lo = unpack2(acc[j].a);
+        zero += 0.f * lo.x + 0.f * lo.y;
+        if constexpr (FOUR) {
+            const float2 hi = unpack2(acc[j].b);
+            zero += 0.f * hi.x + 0.f * hi.y;
+        }
     }
+    if (__any_sync(0xffffffffu, zero != 0.f)) 
+        slice_sums<MODE, C, VS, FLAT, true>(G, A, patch, inside, group, lane, acc);
+    const float rowf = MODE == BWD_ADJOINT ? __ldg(&G.row[0]).y : 1.f;  // else the payload carries it
     unsigned long long skipped = 0;
-    finish_voxel<MODE>(G, A, (long long)patch.iy * G.nx + patch.ix, a, skipped);
+#pragma unroll
+    for (int j = 0; j < C * C; ++j) {
+        if (j) __syncthreads();  // the previous column's sums are read
+        part[threadIdx.x] = acc[j];
+        __syncthreads();
+        const int ix = patch.ix + j % C, iy = patch.iy + j / C;
+        if (group != j % VS || ix >= G.nx || iy >= G.ny) continue;
+        Sums<FOUR> sum = part[lane];
+#pragma unroll
+        for (int g = 1; g < VS; ++g) add_to<FOUR>(sum, part[32 * g + lane]);
+        const float2 lo = unpack2(sum.a);
+        float4 a = make_float4(lo.x * rowf, lo.y * rowf, 0.f, 0.f);
+        if constexpr (FOUR) {
+            const float2 hi = unpack2(sum.b);
+            a.z = hi.x;
+            a.w = hi.y;
+        }
+        finish_voxel<MODE>(G, A, (long long)iy * G.nx + ix, a, skipped);
+    }
     if (FOUR && skipped) atomicAdd(A.skipped, skipped);
 }
 
-template <int VS, bool FLAT>
+template <int C, int VS, bool FLAT>
 static cudaError_t launch_slice(int mode, const Geo& G, const BwdArgs& A, cudaStream_t s) {
-    const int blocks = ((G.nx + 7) / 8) * ((G.ny + 3) / 4);
-    if (mode == BWD_UPDATE) bwd_slice_kernel<BWD_UPDATE, VS, FLAT><<<blocks, 32 * VS, 0, s>>>(G, A);
-    else if (mode == BWD_GRADIENT) bwd_slice_kernel<BWD_GRADIENT, VS, FLAT><<<blocks, 32 * VS, 0, s>>>(G, A);
-    else bwd_slice_kernel<BWD_ADJOINT, VS, FLAT><<<blocks, 32 * VS, 0, s>>>(G, A);
+    const int blocks = ((G.nx + 8 * C - 1) / (8 * C)) * ((G.ny + 4 * C - 1) / (4 * C));
+    if (mode == BWD_UPDATE) bwd_slice_kernel<BWD_UPDATE, C, VS, FLAT><<<blocks, 32 * VS, 0, s>>>(G, A);
+    else if (mode == BWD_GRADIENT) bwd_slice_kernel<BWD_GRADIENT, C, VS, FLAT><<<blocks, 32 * VS, 0, s>>>(G, A);
+    else bwd_slice_kernel<BWD_ADJOINT, C, VS, FLAT><<<blocks, 32 * VS, 0, s>>>(G, A);
     return cudaGetLastError();
 }
 
@@ -554,8 +631,8 @@ cudaError_t launch_backward(int mode, const BwdPlan& P, const Geo& G, const BwdA
 #define DEAM_BWD(SL, VS) \
     if (P.slab == SL && P.vs == VS) return launch_bwd<SL, VS>(mode, G, A, s);
     if (P.slab == 1) {
-        if (P.flat) return P.vs == 4 ? launch_slice<4, true>(mode, G, A, s) : launch_slice<16, true>(mode, G, A, s);
-        return P.vs == 4 ? launch_slice<4, false>(mode, G, A, s) : launch_slice<16, false>(mode, G, A, s);
+        if (P.flat) return P.vs == 8 ? launch_slice<2, 8, true>(mode, G, A, s) : launch_slice<1, 16, true>(mode, G, A, s);
+        return P.vs == 8 ? launch_slice<2, 8, false>(mode, G, A, s) : launch_slice<1, 16, false>(mode, G, A, s);
     }
     DEAM_BWD(2, 4)
     DEAM_BWD(kMidSlab, 1)

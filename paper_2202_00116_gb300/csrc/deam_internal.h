@@ -219,6 +219,9 @@ inline int pick_slab(int nz, int n_rows, double dz, double row_pitch, double sid
 //   11.8 -> 9.9 ms (256^2 x 16: 2048 warps of columns), 11.7 -> 8.5 ms (256^2 x 32);
 //   2 against 1 19.4 -> 18.8 ms (384^2 x 48: 13,824); at 512^2 x 64 (32,768) 1 is
 //   as fast as 2 and 3 % faster than 4.
+//   single slices (slab 1): with four 16 x 8 patches per SM, 2 x 2 columns per thread
+//   and 8 warps of views (4, 8, 16: 0.89, 0.85, 0.90 ms at 512^2); below, one column
+//   per thread and 16 (8: 55 us against 53 at 128^2).
 struct BwdPlan {
     int slab = 2, vs = 4;
     bool flat = false;  // slab 1: all rays lie in the slice
@@ -232,7 +235,7 @@ inline BwdPlan bwd_plan(const deam_geometry& g, bool flat, int sms) {
     if (g.nz == 1 && g.n_rows == 1) {
         p.slab = 1;
         p.flat = flat;
-        p.vs = patches >= 16LL * sms ? 4 : 16;
+        p.vs = patches >= 16LL * sms ? 8 : 16;
         return p;
     }
     const int slab_class = pick_slab(g.nz, g.n_rows, g.dz, g.row_pitch, g.sid, g.sdd);

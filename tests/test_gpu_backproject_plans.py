@@ -68,7 +68,7 @@ GEOMETRIES = {
     "one_row": _geo(nz=9, R=1, V=64, vpr=64),
     "one_column": _geo(nx=1, ny=1, nz=9, dx=60.0, K=33),
     "huge_voxels": _geo(nx=8, ny=7, nz=5, dx=60.0, dz=2.0, K=64),
-    # one slice and one row: sixteen and four warps per patch, in the plane of the
+    # one slice and one row: sixteen and eight warps per patch, in the plane of the
     # source and beside it
     "slice": _geo(nx=45, ny=34, nz=1, R=1, K=90, V=70, vpr=70, feed=0.0),
     "slice_few_views": _geo(nx=20, ny=19, nz=1, R=1, K=31, V=5, vpr=5, feed=0.0),
