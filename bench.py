@@ -343,7 +343,7 @@ def finish_line(args, world, rank, pg, gpu, case, d, mask, c0, samples, ms, valu
     # both projector kernels is the on-chip L1 data path (algorithmic 32 B per
     # Joseph sample against the measured shared-load throughput of this GPU).
     stages = ["layout", "forward", "reduce", "backproject"]
-    avg = {s: kms[i] / max(kn[i], 1) * (2 if s == "layout" else 1) for i, s in enumerate(stages)}
+    avg = {s: kms[i] / max(kn[i], 1) for i, s in enumerate(stages)}
     dom = max(["forward", "backproject"], key=lambda s: avg[s])
     peaks = _peaks()
     sm_max = peaks.get("sm_max_mhz", 2070.0)

@@ -317,7 +317,9 @@ int deam_l1_bandwidth(double *bytes_per_s, void *stream);
  * epilogue, objective reduction, backprojection + update) and accumulates their
  * durations; enable = 0 stops.  deam_kernel_times copies the accumulated
  * milliseconds and launch counts of those four stages into ms[4] and
- * launches[4] (either may be NULL) and, if reset is nonzero, clears them. */
+ * launches[4] (either may be NULL) and, if reset is nonzero, clears them.  The
+ * reduction launches nothing where the forward kernel does it (detectors of one
+ * row, thin volumes). */
 int deam_profile(deam_ctx *ctx, int enable);
 int deam_kernel_times(deam_ctx *ctx, double *ms, long long *launches, int reset);
 

@@ -121,7 +121,7 @@ static cudaError_t dalloc(T** p, size_t n) {
 
 static void free_ctx(deam_ctx* c) {
     void* ptrs[] = {c->view4, c->view_z, c->ip4, c->ipL, c->chan, c->row, c->bowtie, c->dt, c->mask, c->payload,
-                    c->volX, c->volY, c->partial, c->scal, c->hist, c->slab_views, c->skipped, c->c_stage,
+                    c->volX, c->volY, c->partial, c->scal, c->hist, c->slab_views, c->skipped, c->ticket, c->c_stage,
                     c->coef, c->sums, c->fault};
     for (void* p : ptrs)
         if (p) cudaFree(p);
@@ -327,6 +327,7 @@ int deam_init(const deam_geometry* geom, const deam_spectra* spectra, const deam
     G.chan_c0 = (float)((g.n_channels - 1) / 2.0 - g.channel_offset);
     G.inv_dgamma = (float)(1.0 / g.channel_pitch);
     G.fwd_rows = deam::forward_rows(g);
+    G.fwd_narrow = deam::forward_narrow(G, sms);
     ctx->n_fwd_blocks = deam::forward_blocks(G, sms);
     G.vox_reach_mm = (float)(std::max(g.dx, g.dy) * 1.001);
     G.inv_sdd = (float)(1.0 / g.sdd);
@@ -385,6 +386,7 @@ int deam_init(const deam_geometry* geom, const deam_spectra* spectra, const deam
     DEAM_ALLOC(ctx->partial, (size_t)ctx->n_fwd_blocks);
     DEAM_ALLOC(ctx->scal, 4);
     DEAM_ALLOC(ctx->skipped, 1);
+    DEAM_ALLOC(ctx->ticket, 1);
     DEAM_ALLOC(ctx->fault, 2);
     if (spectra->bowtie) DEAM_ALLOC(ctx->bowtie, g.n_channels);
     if (ctx->lambda > 0.0) DEAM_ALLOC(ctx->sums, (size_t)ctx->nvox);
@@ -417,6 +419,7 @@ int deam_init(const deam_geometry* geom, const deam_spectra* spectra, const deam
     }
     A(cudaMemset(ctx->mask, 0, (size_t)ctx->nrays));
     A(cudaMemset(ctx->fault, 0, 2 * sizeof(unsigned int)));
+    A(cudaMemset(ctx->ticket, 0, sizeof(unsigned)));
     A(deam::launch_inplane_table(G, ctx->ip4, ctx->ipL, 0));
     if (e != cudaSuccess) {
         cudaGetLastError();
@@ -573,8 +576,11 @@ static int ray_terms(deam_ctx* ctx, const float2* c, float4* payload, double* F,
     A.mask = ctx->mask_set ? ctx->mask : nullptr;
     A.payload = payload;
     A.fold_rowfac = fold;
+    const bool fused = ctx->G.fwd_rows == 1;  // the forward kernel's last block adds up the objective
+    A.total = fused ? F_dev : nullptr;
+    A.ticket = ctx->ticket;
     CK(deam::launch_forward(ctx->fwd_mode, ctx->G, ctx->S, A, ctx->n_fwd_blocks, s));
-    CK(deam::launch_sum_partials(ctx->partial, ctx->n_fwd_blocks, F_dev, 0, s));
+    if (!fused) CK(deam::launch_sum_partials(ctx->partial, ctx->n_fwd_blocks, F_dev, 0, s));
     if (F) {
         CK(cudaMemcpyAsync(F, F_dev, sizeof(double), cudaMemcpyDeviceToHost, s));
         CK(cudaStreamSynchronize(s));
@@ -643,6 +649,9 @@ int deam_iterate(deam_ctx* ctx, float* c, int n_iter, double* hist, void* stream
     A.mask = ctx->mask_set ? ctx->mask : nullptr;
     A.payload = ctx->payload;
     A.fold_rowfac = 1;
+    A.ticket = ctx->ticket;
+    A.clear = ctx->skipped;  // of the iteration's c-step
+    const bool fused = ctx->G.fwd_rows == 1;  // the forward kernel's last block adds up the objective
     NvtxRange iter_range("deam_iterate");
     for (int it = 0; it < n_iter; ++it) {
         cudaEvent_t* e = ctx->prof ? &ev[(size_t)5 * it] : nullptr;
@@ -654,11 +663,12 @@ int deam_iterate(deam_ctx* ctx, float* c, int n_iter, double* hist, void* stream
         }
         if (e) CK(cudaEventRecord(e[1], s));
         {
-            NvtxRange r("deam.forward");  // Joseph projection + spectral sums + substitution + p-step + F partials
+            NvtxRange r("deam.forward");  // Joseph projection + spectral sums + substitution + p-step + F (partials)
+            A.total = fused ? ctx->hist + it : nullptr;
             CK(deam::launch_forward(ctx->fwd_mode, ctx->G, ctx->S, A, ctx->n_fwd_blocks, s));
         }
         if (e) CK(cudaEventRecord(e[2], s));
-        {
+        if (!fused) {
             NvtxRange r("deam.objective");
             CK(deam::launch_sum_partials(ctx->partial, ctx->n_fwd_blocks, ctx->hist + it, 0, s));
             CK(cudaMemsetAsync(ctx->skipped, 0, sizeof(unsigned long long), s));
@@ -683,7 +693,7 @@ int deam_iterate(deam_ctx* ctx, float* c, int n_iter, double* hist, void* stream
     }
     ctx->skipped_last = (long long)sk;
     if (ctx->prof) {
-        const int nl[4] = {2, 1, 1, 1};
+        const int nl[4] = {1, 1, fused ? 0 : 1, 1};
         for (int it = 0; it < n_iter; ++it)
             for (int j = 0; j < 4; ++j) {
                 float ms = 0.f;

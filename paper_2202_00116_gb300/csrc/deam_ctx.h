@@ -45,6 +45,7 @@ struct deam_ctx {
     double* hist = nullptr;
     int hist_cap = 0;
     int2* slab_views = nullptr;
+    unsigned* ticket = nullptr;  // blocks of the running forward launch that have finished; 0 between launches
     unsigned long long* skipped = nullptr;
     float2* c_stage = nullptr;
     float2* coef = nullptr;  // deam_basis_images coefficients

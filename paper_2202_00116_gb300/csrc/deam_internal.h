@@ -21,6 +21,7 @@ constexpr int kFwdThreads = 256;  // threads per forward block
 struct Geo {
     int nx, ny, nz, V, R, K;
     int fwd_rows;            // rows a forward thread projects at once (forward_rows; host)
+    int fwd_narrow;          // forward blocks of four warps (forward_narrow; host)
     float dx, dy;            // voxel edge lengths (mm)
     float dx_sdd, dy_sdd;    // dx / sdd, dy / sdd
     float dx_dy, dy_dx;      // dx / dy, dy / dx
@@ -146,6 +147,9 @@ struct FwdArgs {
     const float* bowtie;  // [K] (nullable: 1)
     float4* payload;      // FWD_DEAM: [V][R][K] (B~1, B~2, D1, D2)
     double* partial;      // FWD_DEAM: per-block objective; FWD_MAX: per-block max; FWD_COUNT: samples
+    double* total;        // FWD_DEAM with fwd_rows 1: the objective (nullable: the partials alone)
+    unsigned* ticket;     // with total: counts finished blocks; 0 between launches
+    unsigned long long* clear;  // with total: set to 0 (nullable)
     uint8_t* mask_out;    // FWD_MASK
     float threshold;      // FWD_MASK
     int fold_rowfac;      // FWD_DEAM: 1 stores the payload times the row length factor (the
@@ -281,6 +285,11 @@ inline int forward_rows(const deam_geometry& g) {
     return g.n_rows > 4 && g.nz * g.dz >= 2.0 * g.n_rows * g.row_pitch * g.sid / g.sdd ? 8 : 4;
 }
 // Blocks of the persistent forward grid: one resident wave, at most one per tile.
+// Blocks of four warps instead of eight: scans of one row per thread whose blocks of
+// eight are all resident at once, where whole blocks leave some SMs with a third more
+// work than others (128^2 x 360 views, 360 blocks of eight: 33 us, of four 29, of two
+// 29 and longer to add up).
+bool forward_narrow(const Geo& G, int sms);
 int forward_blocks(const Geo& G, int sms);
 cudaError_t launch_forward(int mode, const Geo& G, const Spec& S, const FwdArgs& A, int n_blocks,
                            cudaStream_t s);

@@ -421,6 +421,7 @@ __host__ __device__ __forceinline__ long long ray_tiles(const Geo& G) {
 // fewer views, were 15-40 % slower at 8 rows per thread; at one row they leave
 // warps of a fan-beam scan without a ray).
 constexpr int kBlockViews = kFwdThreads / 32;
+constexpr int kNarrowViews = 4;
 // Whether one of the rows r .. r + rows - 1 has a metal trace at channel k or next to
 // it.  Completing a sinogram reads the prior's line integrals in the trace and at
 // its ends only, so its projection takes these rays (a lane without one waits for
@@ -433,11 +434,39 @@ __device__ __forceinline__ bool near_trace(const Geo& G, const uint8_t* __restri
     return any != 0;
 }
 
+// The block that finishes last adds up the partial objectives, in a fixed order
+// whichever block it is, and clears what the iteration's next kernel counts in: the
+// launches for these two were 7 of the 105 us of an iteration at 128^2.  (Not with
+// rows in groups, whose launches take milliseconds: the code alone made them 3 %
+// slower.)
+template <int NT>
+__device__ __forceinline__ void last_block_total(const FwdArgs& A) {
+    __shared__ bool last;
+    if (threadIdx.x == 0) {
+        __threadfence();  // the partial before the ticket
+        last = atomicAdd(A.ticket, 1u) == gridDim.x - 1;
+    }
+    __syncthreads();
+    if (!last) return;
+    __threadfence();
+    double t = 0.0;
+#pragma unroll 8
+    for (int i = threadIdx.x; i < (int)gridDim.x; i += NT) t += __ldcg(&A.partial[i]);
+    t = block_reduce<NT, double>(t, false);
+    if (threadIdx.x == 0) {
+        *A.total = t;
+        *A.ticket = 0;
+        if (A.clear) *A.clear = 0;
+    }
+}
+
 // Resident blocks per SM: 64, 80 and 128 registers a thread at 1, 4 and 8 rows
 __host__ __device__ constexpr int fwd_min_blocks(int rb) { return rb > 4 ? 2 : rb > 1 ? 3 : 4; }
 
-template <int MODE, int RB>
-__global__ void __launch_bounds__(kFwdThreads, fwd_min_blocks(RB)) fwd_kernel(const Geo G, const Spec S, const FwdArgs A) {
+template <int MODE, int RB, int TV>
+__global__ void __launch_bounds__(32 * TV, fwd_min_blocks(RB) * (kBlockViews / TV)) fwd_kernel(const Geo G, const Spec S,
+                                                                                               const FwdArgs A) {
+    static_assert(RB == 1 || TV == kBlockViews, "rows in groups use blocks of kFwdThreads");
     __shared__ float2 sums[RB > 1 ? RB * kFwdThreads : 1];
     __shared__ SpecTable table;
     if constexpr (RB > 1 && needs_spectrum(MODE)) {
@@ -446,10 +475,10 @@ __global__ void __launch_bounds__(kFwdThreads, fwd_min_blocks(RB)) fwd_kernel(co
     }
     double red = 0.0;  // FWD_DEAM: objective of this thread's rays; FWD_MAX: max l_1
     float redf = 0.f;  // FWD_DEAM_F32: the same in FP32
-    const long long ntiles = ray_tiles<1, kBlockViews, RB>(G);
+    const long long ntiles = ray_tiles<1, TV, RB>(G);
     for (long long t = blockIdx.x; t < ntiles; t += gridDim.x) {
         int v, r, k;
-        if (!ray_of_tile<1, kBlockViews, RB>(G, t, v, r, k)) continue;
+        if (!ray_of_tile<1, TV, RB>(G, t, v, r, k)) continue;
         if (MODE == FWD_LINE && A.mask && !near_trace(G, A.mask, v, r, RB, k)) continue;
         double o;
         if constexpr (RB > 1) o = fwd_rows<MODE, RB>(G, A, v, r, k, sums + threadIdx.x, table, S.e_hi - S.e_lo);
@@ -458,12 +487,14 @@ __global__ void __launch_bounds__(kFwdThreads, fwd_min_blocks(RB)) fwd_kernel(co
         else red = MODE == FWD_MAX ? fmax(red, o) : red + o;
     }
     if (MODE == FWD_DEAM || MODE == FWD_MAX || MODE == FWD_COUNT) {
-        const double b = block_reduce<kFwdThreads, double>(red, MODE == FWD_MAX);
+        const double b = block_reduce<32 * TV, double>(red, MODE == FWD_MAX);
         if (threadIdx.x == 0) A.partial[blockIdx.x] = b;
     } else if (MODE == FWD_DEAM_F32) {
-        const float b = block_reduce<kFwdThreads, float>(redf, false);
+        const float b = block_reduce<32 * TV, float>(redf, false);
         if (threadIdx.x == 0) A.partial[blockIdx.x] = (double)b;
     }
+    if constexpr (RB == 1 && (MODE == FWD_DEAM || MODE == FWD_DEAM_F32))
+        if (A.total) last_block_total<32 * TV>(A);
 }
 
 // ---- regularised c-step (Eqs. 6-7) --------------------------------------
@@ -597,8 +628,10 @@ __global__ void inplane_table_kernel(const Geo G, float4* __restrict__ ip4, floa
 // no bounds tests.  SRC: 0 = float2 image c, 1 = float image m (second
 // component 0), 2 = the constant image (1, 0).
 template <int SRC>
-__global__ void layout_kernel(const float2* __restrict__ c, const float* __restrict__ m, float4* __restrict__ vol,
-                              int axis, int nx, int ny, int nz) {
+__global__ void layout_kernel(const float2* __restrict__ c, const float* __restrict__ m, float4* __restrict__ volX,
+                              float4* __restrict__ volY, int nx, int ny, int nz) {
+    const int axis = blockIdx.y;
+    float4* __restrict__ vol = axis ? volY : volX;
     const int np = axis ? ny : nx, nq = axis ? nx : ny;
     const long long n = (long long)np * (nz + 2) * (nq + 1);
     for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < n;
@@ -775,45 +808,47 @@ static int grid_for(long long n, int threads) {
 
 cudaError_t launch_layout(const float2* c, const float* m, int ones, float4* volX, float4* volY, int nx, int ny,
                           int nz, cudaStream_t s) {
-    for (int axis = 0; axis < 2; ++axis) {
-        const int np = axis ? ny : nx, nq = axis ? nx : ny;
-        const long long n = (long long)np * (nz + 2) * (nq + 1);
-        float4* vol = axis ? volY : volX;
-        const int g = grid_for(n, 256);
-        if (ones) layout_kernel<2><<<g, 256, 0, s>>>(c, m, vol, axis, nx, ny, nz);
-        else if (m) layout_kernel<1><<<g, 256, 0, s>>>(c, m, vol, axis, nx, ny, nz);
-        else layout_kernel<0><<<g, 256, 0, s>>>(c, m, vol, axis, nx, ny, nz);
-    }
+    const long long n = (long long)(nz + 2) * std::max((long long)nx * (ny + 1), (long long)ny * (nx + 1));
+    const dim3 g(grid_for(n, 256), 2);
+    if (ones) layout_kernel<2><<<g, 256, 0, s>>>(c, m, volX, volY, nx, ny, nz);
+    else if (m) layout_kernel<1><<<g, 256, 0, s>>>(c, m, volX, volY, nx, ny, nz);
+    else layout_kernel<0><<<g, 256, 0, s>>>(c, m, volX, volY, nx, ny, nz);
     return cudaGetLastError();
 }
 
 // Resident blocks per SM of the heaviest single-scan forward kernel: the
 // persistent forward grid is this many blocks per SM (one wave; a larger grid
 // of equal-work blocks leaves a partial second wave).
-template <int RB>
+template <int RB, int TV = kBlockViews>
 static long long resident_blocks(const Geo& G, int sms) {
     int a = 0, b = 0;
-    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&a, fwd_kernel<FWD_DEAM, RB>, kFwdThreads, 0) != cudaSuccess ||
-        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&b, fwd_kernel<FWD_DEAM_F32, RB>, kFwdThreads, 0) != cudaSuccess)
-        a = b = fwd_min_blocks(RB);
-    return std::min<long long>(ray_tiles<1, kBlockViews, RB>(G), (long long)sms * std::max(1, std::min(a, b)));
+    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&a, fwd_kernel<FWD_DEAM, RB, TV>, 32 * TV, 0) != cudaSuccess ||
+        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&b, fwd_kernel<FWD_DEAM_F32, RB, TV>, 32 * TV, 0) != cudaSuccess)
+        a = b = fwd_min_blocks(RB) * (kBlockViews / TV);
+    return std::min<long long>(ray_tiles<1, TV, RB>(G), (long long)sms * std::max(1, std::min(a, b)));
+}
+
+bool forward_narrow(const Geo& G, int sms) {
+    return G.fwd_rows == 1 && ray_tiles<1, kBlockViews, 1>(G) <= (long long)sms * fwd_min_blocks(1);
 }
 
 int forward_blocks(const Geo& G, int sms) {
     return (int)(G.fwd_rows == 8   ? resident_blocks<8>(G, sms)
                  : G.fwd_rows == 4 ? resident_blocks<4>(G, sms)
+                 : G.fwd_narrow    ? resident_blocks<1, kNarrowViews>(G, sms)
                                    : resident_blocks<1>(G, sms));
 }
 
-template <int RB>
+template <int RB, int TV = kBlockViews>
 static cudaError_t launch_fwd(int mode, const Geo& G, const Spec& S, const FwdArgs& A, int n_blocks, cudaStream_t s) {
+    constexpr int NT = 32 * TV;
     switch (mode) {
-        case FWD_LINE: fwd_kernel<FWD_LINE, RB><<<n_blocks, kFwdThreads, 0, s>>>(G, S, A); break;
-        case FWD_LINE_G: fwd_kernel<FWD_LINE_G, RB><<<n_blocks, kFwdThreads, 0, s>>>(G, S, A); break;
-        case FWD_DEAM: fwd_kernel<FWD_DEAM, RB><<<n_blocks, kFwdThreads, 0, s>>>(G, S, A); break;
-        case FWD_MASK: fwd_kernel<FWD_MASK, RB><<<n_blocks, kFwdThreads, 0, s>>>(G, S, A); break;
-        case FWD_MAX: fwd_kernel<FWD_MAX, RB><<<n_blocks, kFwdThreads, 0, s>>>(G, S, A); break;
-        case FWD_DEAM_F32: fwd_kernel<FWD_DEAM_F32, RB><<<n_blocks, kFwdThreads, 0, s>>>(G, S, A); break;
+        case FWD_LINE: fwd_kernel<FWD_LINE, RB, TV><<<n_blocks, NT, 0, s>>>(G, S, A); break;
+        case FWD_LINE_G: fwd_kernel<FWD_LINE_G, RB, TV><<<n_blocks, NT, 0, s>>>(G, S, A); break;
+        case FWD_DEAM: fwd_kernel<FWD_DEAM, RB, TV><<<n_blocks, NT, 0, s>>>(G, S, A); break;
+        case FWD_MASK: fwd_kernel<FWD_MASK, RB, TV><<<n_blocks, NT, 0, s>>>(G, S, A); break;
+        case FWD_MAX: fwd_kernel<FWD_MAX, RB, TV><<<n_blocks, NT, 0, s>>>(G, S, A); break;
+        case FWD_DEAM_F32: fwd_kernel<FWD_DEAM_F32, RB, TV><<<n_blocks, NT, 0, s>>>(G, S, A); break;
         default: return cudaErrorInvalidValue;
     }
     return cudaGetLastError();
@@ -821,11 +856,12 @@ static cudaError_t launch_fwd(int mode, const Geo& G, const Spec& S, const FwdAr
 
 cudaError_t launch_forward(int mode, const Geo& G, const Spec& S, const FwdArgs& A, int n_blocks, cudaStream_t s) {
     if (mode == FWD_COUNT) {
-        fwd_kernel<FWD_COUNT, 1><<<n_blocks, kFwdThreads, 0, s>>>(G, S, A);
+        fwd_kernel<FWD_COUNT, 1, kBlockViews><<<n_blocks, kFwdThreads, 0, s>>>(G, S, A);
         return cudaGetLastError();
     }
     return G.fwd_rows == 8   ? launch_fwd<8>(mode, G, S, A, n_blocks, s)
            : G.fwd_rows == 4 ? launch_fwd<4>(mode, G, S, A, n_blocks, s)
+           : G.fwd_narrow    ? launch_fwd<1, kNarrowViews>(mode, G, S, A, n_blocks, s)
                              : launch_fwd<1>(mode, G, S, A, n_blocks, s);
 }
 

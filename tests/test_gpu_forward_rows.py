@@ -82,3 +82,28 @@ def test_objective_equals_one_row_per_thread(pkg):
     H = batch.iterate([c.clone() for c in images], 1)
     np.testing.assert_allclose(H[:, 0], alone, rtol=1e-12)
     batch.close()
+
+
+@pytest.mark.parametrize("name", ["narrow", "wide", "one_row_helical"])
+def test_objective_of_single_rows(pkg, name):
+    # one row per thread: blocks of four and of eight warps, whose last one adds up
+    # the objective; against the batched plan (1e-12), and the same on every call
+    K, V, nz, nx = {"narrow": (31, 9, 1, 20), "wide": (640, 260, 1, 40), "one_row_helical": (70, 333, 7, 24)}[name]
+    geo = synth.Geometry(synth.HELICAL, nx, nx, nz, 4.0, 4.0, 0.75, 0.0, 0.0, 0.0, 570.0, 1040.0, V, V, 0.3,
+                         0.6 if nz > 1 else 0.0, -0.3 if nz > 1 else 0.0, 1, 0.75 * 1040.0 / 570.0, K,
+                         synth.fan_pitch(nx * 2.0, 570.0, K), 0.25, 0.0)
+    s = pkg.from_case(_case(geo))
+    gen = torch.Generator().manual_seed(1)
+    s.set_data((1e5 * torch.rand((2, V, 1, K), generator=gen)).cuda())
+    c = (0.3 * torch.rand((nz, nx, nx, 2), generator=gen)).cuda()
+    F = [s.objective(c) for _ in range(3)]
+    assert F[0] == F[1] == F[2]
+    H = s.iterate(c.clone(), 3)
+    info = s.info()
+    batch = pkg.DeamBatch([s], autotune=False)
+    B = batch.iterate([c.clone()], 3)
+    np.testing.assert_allclose(B[0, 0], F[0], rtol=1e-12)
+    np.testing.assert_allclose(H[0], F[0], rtol=1e-12)
+    np.testing.assert_allclose(H, B[0], rtol=1e-7)
+    assert np.array_equal(s.iterate(c.clone(), 3), H) and s.info() == info   # skipped voxels counted anew
+    batch.close()
