@@ -328,7 +328,7 @@ int deam_init(const deam_geometry* geom, const deam_spectra* spectra, const deam
     G.inv_dgamma = (float)(1.0 / g.channel_pitch);
     G.fwd_rows = deam::forward_rows(g);
     G.fwd_narrow = deam::forward_narrow(G, sms);
-    ctx->n_fwd_blocks = deam::forward_blocks(G, sms);
+    ctx->n_fwd_blocks = deam::forward_blocks(G);
     G.vox_reach_mm = (float)(std::max(g.dx, g.dy) * 1.001);
     G.inv_sdd = (float)(1.0 / g.sdd);
 
@@ -769,9 +769,10 @@ int deam_penalty(deam_ctx* ctx, const float* c, double* R, void* stream) {
     NEED_DEVICE(c, "c");
     cudaStream_t s = (cudaStream_t)stream;
     const deam_geometry& g = ctx->geo;
+    const int blocks = std::min(ctx->n_fwd_blocks, 152 * 8);  // one wave over the voxels
     CK(deam::launch_penalty((const float2*)c, g.nx, g.ny, g.nz, (float)g.dx, (float)g.dy, (float)g.dz,
-                            (float)ctx->lambda, (float)ctx->delta, ctx->partial, ctx->n_fwd_blocks, s));
-    CK(deam::launch_sum_partials(ctx->partial, ctx->n_fwd_blocks, ctx->scal + 2, 0, s));
+                            (float)ctx->lambda, (float)ctx->delta, ctx->partial, blocks, s));
+    CK(deam::launch_sum_partials(ctx->partial, blocks, ctx->scal + 2, 0, s));
     CK(cudaMemcpyAsync(R, ctx->scal + 2, sizeof(double), cudaMemcpyDeviceToHost, s));
     CK(cudaStreamSynchronize(s));
     return DEAM_OK;

@@ -284,13 +284,13 @@ inline int forward_rows(const deam_geometry& g) {
     if (!(w < 2048.0)) return 1;
     return g.n_rows > 4 && g.nz * g.dz >= 2.0 * g.n_rows * g.row_pitch * g.sid / g.sdd ? 8 : 4;
 }
-// Blocks of the persistent forward grid: one resident wave, at most one per tile.
 // Blocks of four warps instead of eight: scans of one row per thread whose blocks of
 // eight are all resident at once, where whole blocks leave some SMs with a third more
 // work than others (128^2 x 360 views, 360 blocks of eight: 33 us, of four 29, of two
 // 29 and longer to add up).
 bool forward_narrow(const Geo& G, int sms);
-int forward_blocks(const Geo& G, int sms);
+// Blocks of the forward grid: one per ray tile.
+int forward_blocks(const Geo& G);
 cudaError_t launch_forward(int mode, const Geo& G, const Spec& S, const FwdArgs& A, int n_blocks,
                            cudaStream_t s);
 cudaError_t launch_backward(int mode, const BwdPlan& P, const Geo& G, const BwdArgs& A, cudaStream_t s);

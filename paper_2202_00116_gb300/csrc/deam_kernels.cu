@@ -664,6 +664,7 @@ __global__ void __launch_bounds__(256) sum_partials_kernel(const double* __restr
                                                            int do_max) {
     __shared__ double sh[256];
     double v = do_max ? -INFINITY : 0.0;
+#pragma unroll 8
     for (int i = threadIdx.x; i < n; i += 256) v = do_max ? fmax(v, p[i]) : v + p[i];
     sh[threadIdx.x] = v;
     __syncthreads();
@@ -816,27 +817,20 @@ cudaError_t launch_layout(const float2* c, const float* m, int ones, float4* vol
     return cudaGetLastError();
 }
 
-// Resident blocks per SM of the heaviest single-scan forward kernel: the
-// persistent forward grid is this many blocks per SM (one wave; a larger grid
-// of equal-work blocks leaves a partial second wave).
-template <int RB, int TV = kBlockViews>
-static long long resident_blocks(const Geo& G, int sms) {
-    int a = 0, b = 0;
-    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&a, fwd_kernel<FWD_DEAM, RB, TV>, 32 * TV, 0) != cudaSuccess ||
-        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&b, fwd_kernel<FWD_DEAM_F32, RB, TV>, 32 * TV, 0) != cudaSuccess)
-        a = b = fwd_min_blocks(RB) * (kBlockViews / TV);
-    return std::min<long long>(ray_tiles<1, TV, RB>(G), (long long)sms * std::max(1, std::min(a, b)));
-}
-
 bool forward_narrow(const Geo& G, int sms) {
     return G.fwd_rows == 1 && ray_tiles<1, kBlockViews, 1>(G) <= (long long)sms * fwd_min_blocks(1);
 }
 
-int forward_blocks(const Geo& G, int sms) {
-    return (int)(G.fwd_rows == 8   ? resident_blocks<8>(G, sms)
-                 : G.fwd_rows == 4 ? resident_blocks<4>(G, sms)
-                 : G.fwd_narrow    ? resident_blocks<1, kNarrowViews>(G, sms)
-                                   : resident_blocks<1>(G, sms));
+// A block per ray tile, handed out in order as SMs become free: the tiles in flight
+// are neighbours and share the volume in L1 and L2.  One wave of blocks that walk the
+// tiles in strides drifts apart (512^2 x 64, 5 rotations: 63.3 against 52.1 ms, 384^2 x
+// 48 9.0 against 7.6, 301 x 277 x 37 with 15 rows 2.71 against 2.17).
+int forward_blocks(const Geo& G) {
+    const long long n = G.fwd_rows == 8   ? ray_tiles<1, kBlockViews, 8>(G)
+                        : G.fwd_rows == 4 ? ray_tiles<1, kBlockViews, 4>(G)
+                        : G.fwd_narrow    ? ray_tiles<1, kNarrowViews, 1>(G)
+                                          : ray_tiles<1, kBlockViews, 1>(G);
+    return (int)std::min<long long>(n, 1LL << 30);  // (more: the blocks go on to further tiles)
 }
 
 template <int RB, int TV = kBlockViews>
