@@ -329,8 +329,8 @@ int deam_kernel_times(deam_ctx *ctx, double *ms, long long *launches, int reset)
  * deam_set_metal_mask) called; contexts must outlive the batch, live on the
  * current device, and not be used by other calls while the batch iterates.
  * One iteration of the batch is the MAR-DEAM iteration of deam_iterate for
- * every scan, run as one persistent forward launch and one persistent
- * backprojection launch over the work of all scans, captured once in a CUDA
+ * every scan, run as one forward launch and one backprojection launch (per
+ * slab class) over the work of all scans, captured once in a CUDA
  * graph and replayed.  autotune = 0 runs the persistent plan with default
  * shapes, 2 the per-scan plan (below) without tuning.  With autotune = 1 the first deam_batch_iterate times the
  * candidate ray-tile shapes (32 channels x rows x views) and backprojection

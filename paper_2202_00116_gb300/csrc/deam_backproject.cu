@@ -596,7 +596,7 @@ __global__ void __launch_bounds__(kBwdThreads, 5) bwd_kernel(const Geo G, const 
     bwd_tile<MODE, SLAB, TX, TY, VS>(G, A, acc, bx, by, b / nty);
 }
 
-// Batched scans: one persistent launch walks the column tiles x slabs of every
+// Batched scans: one launch takes the column tiles x slabs of every
 // scan of a slab class; each work item finds its scan by binary search in the
 // prefix sums of tile counts.
 // (the scan's descriptors are held in registers, hence one block per SM less)
@@ -653,16 +653,6 @@ long long backward_tiles(int shape, const Geo& G) {
 
 #define DEAM_BWD_BATCH_SHAPES(X) \
     X(0, 2, 16, 8) X(1, 2, 32, 4) X(2, 8, 16, 8) X(3, 8, 32, 4) X(4, 16, 16, 8) X(5, 16, 32, 4)
-
-int backward_batch_blocks_per_sm(int shape) {
-    int nb = 1;
-#define X(I, SL, TX, TY) \
-    if (shape == I) cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, bwd_batch_kernel<SL, TX, TY>, TX * TY, 0);
-    DEAM_BWD_BATCH_SHAPES(X)
-#undef X
-    return nb > 0 ? nb : 1;
-}
-
 
 cudaError_t launch_backward_batch(int shape, const BatchDesc& B, int grid, cudaStream_t s) {
 #define X(I, SL, TX, TY) \

@@ -1,8 +1,8 @@
 // Batched MAR-DEAM: many independent scans (each a deam_ctx with its data and
 // metal mask set) iterated together.  One iteration is a fixed set of launches
-// whatever the number of scans: the per-scan projector layouts, one persistent
+// whatever the number of scans: the per-scan projector layouts, one
 // forward launch over the ray tiles of every scan, one launch reducing every
-// scan's objective, one persistent backprojection launch per slab class (2, 8
+// scan's objective, one backprojection launch per slab class (2, 8
 // or 16 slices, from each scan's geometry) over the column tiles of its scans,
 // and an iteration counter.  The sequence is captured once in a CUDA graph and
 // replayed per iteration.  The ray-tile shape of the forward launch and the
@@ -30,6 +30,9 @@ constexpr int kNF = 3;  // forward ray-tile shapes (deam::kFwdShapes)
 constexpr int kNB = deam::kNumBwdShapes;  // backprojection shapes (deam::kBwdShapes)
 constexpr int kSlabs[3] = {2, 8, 16};     // slab classes
 
+// A block per work item, handed out in order as SMs become free.
+int grid_of(long long items) { return (int)std::min(std::max(items, 1LL), 1LL << 30); }
+
 }  // namespace
 
 struct deam_batch {
@@ -54,7 +57,7 @@ struct deam_batch {
     bool tuned = false;
     float tune_fwd_ms[kNF] = {0, 0, 0}, tune_bwd_ms[kNB] = {0, 0, 0, 0, 0, 0};
     int fgrid[kNF] = {}, bgrid[kNB] = {};
-    int plan = 0;                    // 0: persistent launches over all scans, 1: per-scan launches on graph branches
+    int plan = 0;                    // 0: one launch per stage over all scans, 1: per-scan launches on graph branches
     int min_plan = 0;                // 1 when a scan asks for the plain-FP32 forward (plan 0 has only the compensated one)
     float tune_plan_ms[2] = {0, 0};
     long long* soff = nullptr;       // [n][2] = {0, forward blocks of scan i}: per-scan objective ranges
@@ -196,7 +199,7 @@ static int tune(deam_batch* b, float* const* c) {
 }
 
 // Record one iteration of the whole batch on the capturing stream b->cs.
-// plan 0: the persistent batched kernels; plan 1: every scan's own kernels
+// plan 0: the batched kernels; plan 1: every scan's own kernels
 // (the single-scan launches of deam_iterate) on a graph branch of its own.
 static int record_iteration(deam_batch* b, float* const* c, int plan) {
     cudaStream_t s = b->cs;
@@ -211,7 +214,7 @@ static int record_iteration(deam_batch* b, float* const* c, int plan) {
             e = deam::launch_sum_ranges(b->partial, b->foff[b->fshape], b->n, b->hist, b->counter, b->hist_cap, s);
         for (int i = 0; i < b->n && e == cudaSuccess; ++i)
             e = cudaMemsetAsync(b->ctx[i]->skipped, 0, sizeof(unsigned long long), s);
-        for (int cl = 0; cl < 3 && e == cudaSuccess; ++cl)  // one persistent launch per slab class
+        for (int cl = 0; cl < 3 && e == cudaSuccess; ++cl)  // one launch per slab class
             if (b->bshape[cl] >= 0)
                 e = deam::launch_backward_batch(b->bshape[cl], desc(b, b->fshape, b->bshape[cl]),
                                                 b->bgrid[b->bshape[cl]], s);
@@ -378,8 +381,6 @@ int deam_batch_create(deam_ctx* const* ctxs, int n, int autotune, deam_batch** o
     }
     std::vector<long long> off(n + 1);
     long long maxf = 0;
-    int sms = 152;
-    cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
     cudaError_t e = cudaSuccess;
     auto A = [&](cudaError_t r) {
         if (e == cudaSuccess) e = r;
@@ -399,7 +400,7 @@ int deam_batch_create(deam_ctx* const* ctxs, int n, int autotune, deam_batch** o
         A(cudaMalloc((void**)&b->foff[fs], sizeof(long long) * (n + 1)));
         if (e == cudaSuccess)
             A(cudaMemcpy(b->foff[fs], off.data(), sizeof(long long) * (n + 1), cudaMemcpyHostToDevice));
-        b->fgrid[fs] = sms * deam::forward_batch_blocks_per_sm(fs);
+        b->fgrid[fs] = grid_of(off[n]);
     }
     A(cudaMalloc((void**)&b->partial, sizeof(double) * std::max<long long>(maxf, 1)));
     std::vector<int> cls(n);
@@ -439,7 +440,7 @@ int deam_batch_create(deam_ctx* const* ctxs, int n, int autotune, deam_batch** o
             a.skipped = ctxs[i]->skipped;
             deam::set_penalty_args(ctxs[i], a);
         }
-        b->bgrid[bs] = sms * deam::backward_batch_blocks_per_sm(bs);
+        b->bgrid[bs] = grid_of(off[n]);
         if (off[n] > 0 && (b->bshape[cl] < 0 || deam::kBwdShapes[bs][1] == 16)) b->bshape[cl] = bs;  // default 16x8
         b->class_tiles[cl] = off[n];
     }

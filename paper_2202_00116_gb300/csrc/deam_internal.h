@@ -204,7 +204,7 @@ constexpr int kBwdShapes[kNumBwdShapes][3] = {{2, 16, 8}, {2, 32, 4}, {8, 16, 8}
                                               {8, 32, 4}, {16, 16, 8}, {16, 32, 4}};  // (slab, tx, ty)
 // Slab class of the gather backprojection for a scan: 2 for one or two
 // slices, 8 when a detector row covers at most 2/3 of a slice (several rows
-// per slice), else 16.  The batched persistent launches use the class as their
+// per slice), else 16.  The batched launches use the class as their
 // slab depth; a single-scan context runs its own plan (bwd_plan).
 inline int pick_slab(int nz, int n_rows, double dz, double row_pitch, double sid, double sdd) {
     if (nz <= 2) return 2;
@@ -252,8 +252,6 @@ inline BwdPlan bwd_plan(const deam_geometry& g, bool flat, int sms) {
 }
 long long forward_tiles(int shape, const Geo& G);
 long long backward_tiles(int shape, const Geo& G);
-int forward_batch_blocks_per_sm(int shape);
-int backward_batch_blocks_per_sm(int shape);
 cudaError_t launch_forward_batch(int shape, const BatchDesc& B, int grid, cudaStream_t s);
 cudaError_t launch_backward_batch(int shape, const BatchDesc& B, int grid, cudaStream_t s);
 // out[i * stride + *counter] = sum of partial[off[i] .. off[i+1]) (fixed order)
