@@ -46,11 +46,11 @@ L1_BYTES_PER_SAMPLE = 32.0
 # one-rotation cut of this scan (6.484e9 samples per launch; the commands are
 # in profiles/); traffic grows with the views, so it is scaled by the sample
 # count of the measured launch.  Kernels without a capture of their current
-# build are absent (traffic null): the backprojection's capture (3.04 GB per
-# 6.4845e9 samples) predates its row loop losing its unroll.
-DRAM_BYTES_PER_SAMPLE = {"fwd_kernel<FWD_DEAM>": (1.9193e9 + 0.2392e9) / 6.4845e9}
+# build are absent (traffic null).
+DRAM_BYTES_PER_SAMPLE = {"fwd_kernel<FWD_DEAM>": (2.3191e9 + 0.2350e9) / 6.4845e9,
+                         "bwd_kernel<1,16>": (1.2712e9 + 0.1394e9) / 6.4845e9}
 # L1/TEX utilisation of the same kernels in those captures.
-L1_BUSY = {"fwd_kernel<FWD_DEAM>": 0.682}
+L1_BUSY = {"fwd_kernel<FWD_DEAM>": 0.700, "bwd_kernel<1,16>": 0.690}
 
 
 def _peaks():
@@ -351,10 +351,10 @@ def finish_line(args, world, rank, pg, gpu, case, d, mask, c0, samples, ms, valu
     hbm_src = "MEASURED_PEAKS.json hbm_gbs (of measured)"
     if hbm is None:
         hbm, hbm_src = 6800.0, "profiling recipe fallback 6.8 TB/s (of fallback)"
-    # the library's slab depth for this scan (2 for one or two slices, 8 for thin
-    # rows, else 13)
+    # the library's slab depth for this scan (2 for one or two slices, 11 for thin
+    # rows, else 16)
     slab = (2 if geo.nz <= 2 else
-            8 if (geo.n_rows == 1 or geo.dz >= 1.5 * geo.row_pitch * geo.sid / geo.sdd) else 13)
+            11 if (geo.n_rows == 1 or geo.dz >= 1.5 * geo.row_pitch * geo.sid / geo.sdd) else 16)
     kname = {"forward": "fwd_kernel<FWD_DEAM>", "backproject": f"bwd_kernel<1,{slab}>"}[dom]
     nvox, nrays = geo.n_voxels, geo.n_rays
     # compulsory bytes per launch: forward reads c (via its two layouts, 8 B per

@@ -27,8 +27,8 @@ namespace deam {
 // payload gathers with the 20 warps per SM that 96 registers allow, the L1 data
 // path being 60-70 % busy.  One ray at a time (two views abreast) cost twice the
 // shared-memory traffic, half the loads in flight and 70 instead of 31
-// instructions per (column, ray, row): 37.4 -> 22.9 ms on one rotation of the
-// 512^2 x 64 scan, 20.5 -> 8.6 ms on one of the 256^2 x 32 scan.  Measured and
+// instructions per (column, ray, row): 37.4 -> 23.3 ms on one rotation of the
+// 512^2 x 64 scan, 20.5 -> 8.5 ms on one of the 256^2 x 32 scan.  Measured and
 // slower: sums in registers with the slices unrolled (37.5 ms on the first),
 // four views per turn (29-50 ms), first moments of the rays' heights instead of
 // each ray's own weights (32.6 ms, and no longer the forward's weights).

@@ -266,11 +266,11 @@ cudaError_t launch_layout(const float2* c, const float* m, int ones, float4* vol
 //   1: one row, or a volume or cone too large for its floor and step tests
 //      (indices below 2^21, heights below 2048 slices).
 //   8: a volume at least twice as high as the detector covers at the axis: most
-//      rows meet it along the whole ray.  Against 4 rows, one launch: 11.5 / 12.9
-//      ms on a rotation of 512^2 x 64, 9.2 / 9.7 ms at 384^2 x 48, 3.1 / 3.3 ms on
-//      a rotation of 256^2 x 32 (against one row 15.4, 14.0 and 5.4 ms).
+//      rows meet it along the whole ray.  Against 4 rows, one launch: 10.5 / 10.6
+//      ms on a rotation of 512^2 x 64, 7.6 / 7.7 ms at 384^2 x 48, 3.0 / 3.1 ms on
+//      a rotation of 256^2 x 32 (one row, in one wave of blocks: 15.4, 14.0, 5.4).
 //   4: thinner volumes, where rows in larger groups are carried along outside
-//      (256^2 x 16, 1440 views: 5.0 ms against 5.9 with 8 and 6.3 with 1), and
+//      (256^2 x 16, 1440 views: 4.4 ms against 5.0 with 8; one row 6.3), and
 //      detectors of few rows.
 inline int forward_rows(const deam_geometry& g) {
     if (g.n_rows < 2 || g.nx >= (1 << 21) || g.ny >= (1 << 21) || g.nz >= 2048) return 1;
