@@ -403,7 +403,10 @@ __device__ __forceinline__ void bwd_tile(const Geo& G, const BwdArgs& A, Sums<MO
                             Sums<FOUR> lo = acc[s * NT], hi = acc[(s + 1) * NT];
 #pragma unroll
                             for (int g = 0; g < G_; ++g) {
-                                const float x = row_fz(sza, om, a.t[g]) - fs, y = row_fz(szb, om, b.t[g]) - fs;
+                                // rounded down: a height just below slice 0 is less than 1 above
+                                // slice -1 (all other differences are exact)
+                                const float x = __fsub_rd(row_fz(sza, om, a.t[g]), fs);
+                                const float y = __fsub_rd(row_fz(szb, om, b.t[g]), fs);
                                 if (x >= 0.f && x < 1.f) add_sample<FOUR>(lo, hi, x, a.c[g] * rowf, P[g]);
                                 if (y >= 0.f && y < 1.f) add_sample<FOUR>(lo, hi, y, b.c[g] * rowf, Q[g]);
                             }
