@@ -406,24 +406,37 @@ int complete(deam_ctx* ctx, const float* p, const float* prior, int pstride, int
     return DEAM_OK;
 }
 
+// Bytes of shared memory of ramp_kernel: the taps, and each row of K channels.
+struct RampShared {
+    size_t taps, row;
+};
+RampShared ramp_shared(int K, int ns) {
+    const size_t cell = sizeof(float) * ns;
+    const int half = (K + 1) / 2, taps = (K / 2 + 3) / 4 * 4, len = 2 * (taps + 8) + (half + 3) / 4 * 4;
+    return {taps * cell, 2 * (size_t)len * cell};
+}
+
 template <int NS>
 cudaError_t filter(deam_ctx* ctx, const float* p, const float* chanw, const float* conew, const float* ker, float* q,
                    cudaStream_t s) {
     const int K = ctx->geo.n_channels, R = ctx->geo.n_rows;
     const long long nrows = (long long)ctx->geo.n_views * R;
-    const int half = (K + 1) / 2, taps = (K / 2 + 3) / 4 * 4, len = 2 * (taps + 8) + (half + 3) / 4 * 4;
-    const size_t cell = sizeof(float) * NS, row = 2 * (size_t)len * cell;
+    const RampShared m = ramp_shared(K, NS);
     // rows per block: outputs (in fours) for half as many threads again, as far as
     // 48 KB hold their rows, so that the threads with short windows take a second one
     // (two rows of 672 channels; one row, 0.3 to 0.7 ms slower of 15.5 for the whole
     // initialisation); a long row may need more, by opt-in (3072 channels of two
-    // spectra: 87 KB)
-    const int fours = 2 * ((half + 3) / 4);
-    const size_t room = 48 * 1024 > taps * cell + row ? 48 * 1024 - taps * cell : row;
-    const int per = (int)std::min<size_t>(std::max(1, 384 / fours), room / row);
-    const size_t sm = taps * cell + per * row;
+    // spectra: 86 KB)
+    const int fours = 2 * (((K + 1) / 2 + 3) / 4);
+    const size_t room = 48 * 1024 > m.taps + m.row ? 48 * 1024 - m.taps : m.row;
+    const int per = (int)std::min<size_t>(std::max(1, 384 / fours), room / m.row);
+    const size_t sm = m.taps + per * m.row;
     if (sm > 48 * 1024) {
-        const cudaError_t e = cudaFuncSetAttribute(ramp_kernel<NS>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
+        // the limit is the kernel's, not this call's: always the longest row's, so that
+        // calls of several threads do not lower it for one another
+        const RampShared most = ramp_shared(kMaxFbpChannels, NS);
+        const cudaError_t e = cudaFuncSetAttribute(ramp_kernel<NS>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                                   (int)(most.taps + most.row));
         if (e != cudaSuccess) return e;
     }
     const int blocks = (int)std::min<long long>((nrows + per - 1) / per, 1LL << 20);
