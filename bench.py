@@ -47,10 +47,22 @@ L1_BYTES_PER_SAMPLE = 32.0
 # in profiles/); traffic grows with the views, so it is scaled by the sample
 # count of the measured launch.  Kernels without a capture of their current
 # build are absent (traffic null).
-DRAM_BYTES_PER_SAMPLE = {"fwd_kernel<FWD_DEAM>": (2.3191e9 + 0.2350e9) / 6.4845e9,
-                         "bwd_kernel<1,16>": (1.2712e9 + 0.1394e9) / 6.4845e9}
+DRAM_BYTES_PER_SAMPLE = {"fwd_kernel<FWD_DEAM,8>": (2.3191e9 + 0.2350e9) / 6.4845e9,
+                         "bwd_kernel<1,16,1>": (1.2712e9 + 0.1394e9) / 6.4845e9}
 # L1/TEX utilisation of the same kernels in those captures.
-L1_BUSY = {"fwd_kernel<FWD_DEAM>": 0.700, "bwd_kernel<1,16>": 0.690}
+L1_BUSY = {"fwd_kernel<FWD_DEAM,8>": 0.700, "bwd_kernel<1,16,1>": 0.690}
+
+
+def kernel_name(stage, plan):
+    """Name of the kernel that a scan of this plan (Deam.kernel_plan) runs in a stage:
+    the forward with its rows per thread, the backprojection with its slab depth, the
+    warps that share a column's views and, but for the usual four, its rays per turn."""
+    if stage == "forward":
+        return f"fwd_kernel<FWD_DEAM,{plan['fwd_rows']}>"
+    if plan["bwd_slab"] == 1:
+        return f"bwd_slice_kernel<1,{plan['bwd_groups']}>"
+    rays = "" if plan["bwd_rays"] == 4 else f",{plan['bwd_rays']}"
+    return f"bwd_kernel<1,{plan['bwd_slab']},{plan['bwd_groups']}{rays}>"
 
 
 def _peaks():
@@ -351,11 +363,7 @@ def finish_line(args, world, rank, pg, gpu, case, d, mask, c0, samples, ms, valu
     hbm_src = "MEASURED_PEAKS.json hbm_gbs (of measured)"
     if hbm is None:
         hbm, hbm_src = 6800.0, "profiling recipe fallback 6.8 TB/s (of fallback)"
-    # the library's slab depth for this scan (2 for one or two slices, 11 for thin
-    # rows, else 16)
-    slab = (2 if geo.nz <= 2 else
-            11 if (geo.n_rows == 1 or geo.dz >= 1.5 * geo.row_pitch * geo.sid / geo.sdd) else 16)
-    kname = {"forward": "fwd_kernel<FWD_DEAM>", "backproject": f"bwd_kernel<1,{slab}>"}[dom]
+    kname = kernel_name(dom, gpu.kernel_plan())
     nvox, nrays = geo.n_voxels, geo.n_rays
     # compulsory bytes per launch: forward reads c (via its two layouts, 8 B per
     # voxel each way counted once: 16 B/voxel), d~ (8 B/ray) and the mask

@@ -318,10 +318,23 @@ int deam_l1_bandwidth(double *bytes_per_s, void *stream);
  * durations; enable = 0 stops.  deam_kernel_times copies the accumulated
  * milliseconds and launch counts of those four stages into ms[4] and
  * launches[4] (either may be NULL) and, if reset is nonzero, clears them.  The
- * reduction launches nothing where the forward kernel does it (detectors of one
- * row, thin volumes). */
+ * reduction launches nothing where the forward kernel does it (plans of one row
+ * per thread). */
 int deam_profile(deam_ctx *ctx, int enable);
 int deam_kernel_times(deam_ctx *ctx, double *ms, long long *launches, int reset);
+
+/* How the kernels of a context split their work, chosen by deam_init from the
+ * geometry. */
+typedef struct deam_plan {
+    int fwd_rows;   /* detector rows that a thread of the forward projection takes */
+    int bwd_slab;   /* slices that a block of the backprojection takes (1: the kernel of single slices) */
+    int bwd_groups; /* warps that share the views of a column */
+    int bwd_rays;   /* rays of a view that one turn of the backprojection takes */
+    int reserved[4];
+} deam_plan;
+
+/* The plan of the context (host memory). */
+int deam_kernel_plan(const deam_ctx *ctx, deam_plan *plan);
 
 /* ---- Batched scans ------------------------------------------------------
  * Many independent scans of uneven size and view count, iterated together.

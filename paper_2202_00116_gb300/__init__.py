@@ -60,6 +60,11 @@ class deam_mar_params(C.Structure):
                 ("prior_spectrum", C.c_int), ("prior_smooth", C.c_int), ("reserved", C.c_int * 6)]
 
 
+class deam_plan(C.Structure):
+    _fields_ = [("fwd_rows", C.c_int), ("bwd_slab", C.c_int), ("bwd_groups", C.c_int), ("bwd_rays", C.c_int),
+                ("reserved", C.c_int * 4)]
+
+
 class DeamError(RuntimeError):
     def __init__(self, code, msg):
         super().__init__(f"deam error {code}: {msg}")
@@ -71,7 +76,7 @@ EXPORTS = ["deam_init", "deam_set_data", "deam_set_metal_mask", "deam_get_metal_
            "deam_backproject", "deam_ray_terms", "deam_iterate", "deam_objective", "deam_info",
            "deam_gradient", "deam_backprojected_sums", "deam_penalty", "deam_basis_images", "deam_vmi",
            "deam_kvp_images", "deam_count_samples",
-           "deam_profile", "deam_kernel_times", "deam_l1_bandwidth", "deam_bounds_checked", "deam_bounds_inject", "deam_log_sinogram", "deam_complete_trace", "deam_fbp",
+           "deam_profile", "deam_kernel_times", "deam_kernel_plan", "deam_l1_bandwidth", "deam_bounds_checked", "deam_bounds_inject", "deam_log_sinogram", "deam_complete_trace", "deam_fbp",
            "deam_mar_init", "deam_batch_create",
            "deam_batch_iterate", "deam_batch_info", "deam_batch_destroy", "deam_objective_noalloc",
            "deam_destroy", "deam_last_error"]
@@ -109,6 +114,7 @@ def lib():
             "deam_bounds_checked": [],
             "deam_bounds_inject": [vp, vp],
             "deam_kernel_times": [vp, pd, C.POINTER(C.c_longlong), i],
+            "deam_kernel_plan": [vp, C.POINTER(deam_plan)],
             "deam_log_sinogram": [vp, C.c_double, vp, vp],
             "deam_complete_trace": [vp, vp, vp, i, C.c_double, vp, vp],
             "deam_fbp": [vp, vp, i, vp, vp],
@@ -410,6 +416,12 @@ class Deam:
         n = (C.c_longlong * 4)()
         _check(lib().deam_kernel_times(self._h, ms, n, int(bool(reset))))
         return list(ms), list(n)
+
+    def kernel_plan(self):
+        """How the kernels split their work on this scan (deam_kernel_plan)."""
+        p = deam_plan()
+        _check(lib().deam_kernel_plan(self._h, C.byref(p)))
+        return {k: getattr(p, k) for k, _ in deam_plan._fields_ if k != "reserved"}
 
     def close(self):
         """Release the context (raises DeamError while a live DeamBatch holds it)."""

@@ -911,4 +911,15 @@ int deam_kernel_times(deam_ctx* ctx, double* ms, long long* launches, int reset)
     return DEAM_OK;
 }
 
+int deam_kernel_plan(const deam_ctx* ctx, deam_plan* plan) {
+    if (!ctx) return fail(DEAM_ERR_ARG, "null context");
+    if (!plan) return fail(DEAM_ERR_ARG, "plan must not be NULL");
+    *plan = deam_plan{};
+    plan->fwd_rows = ctx->G.fwd_rows;
+    plan->bwd_slab = ctx->bwd.slab;
+    plan->bwd_groups = ctx->bwd.vs;
+    plan->bwd_rays = ctx->bwd.slab > 1 ? deam::kRaysPerView : 1;
+    return DEAM_OK;
+}
+
 }  // extern "C"

@@ -33,11 +33,6 @@ namespace deam {
 // four views per turn (29-50 ms), first moments of the rays' heights instead of
 // each ray's own weights (32.6 ms, and no longer the forward's weights).
 constexpr int kBwdThreads = 128;
-// Rays of a view that one turn of the row loop takes (more rays: more turns).
-// Four at 5 blocks of 128 threads per SM; three at 6 blocks are as fast at 2.6
-// rays per view and 8 % slower at 3.5 (384^2 x 48 on 816 channels).
-constexpr int kRaysPerView = 4;
-
 
 // A ray's data, or the sums of a voxel: (b~_1, b~_2) and, for the c-step, also
 // (delta_1, delta_2).  The gradient carries the second pair alone, the plain
