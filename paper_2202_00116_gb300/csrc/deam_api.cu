@@ -333,7 +333,7 @@ int deam_init(const deam_geometry* geom, const deam_spectra* spectra, const deam
     G.domega = (float)(g.row_pitch / g.dz);
     G.chan_c0 = (float)((g.n_channels - 1) / 2.0 - g.channel_offset);
     G.inv_dgamma = (float)(1.0 / g.channel_pitch);
-    G.fwd_rows = deam::forward_rows(g);
+    G.fwd_rows = deam::forward_rows(g, sms);
     G.fwd_narrow = deam::forward_narrow(G, sms);
     ctx->n_fwd_blocks = deam::forward_blocks(G);
     G.vox_reach_mm = (float)(std::max(g.dx, g.dy) * 1.001);

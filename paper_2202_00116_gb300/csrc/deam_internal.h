@@ -266,26 +266,8 @@ cudaError_t launch_counter_inc(int* counter, cudaStream_t s);
 cudaError_t launch_inplane_table(const Geo& G, float4* ip4, float* ipL, cudaStream_t s);
 cudaError_t launch_layout(const float2* c, const float* m, int ones, float4* volX, float4* volY,
                           int nx, int ny, int nz, cudaStream_t s);
-// Detector rows that a thread of the forward kernel projects at once (fwd_rows).
-//   1: one row, or a volume or cone too large for its floor and step tests
-//      (indices below 2^21, heights below 2048 slices).
-//   8: a volume at least twice as high as the detector covers at the axis: most
-//      rows meet it along the whole ray.  Against 4 rows, one launch: 10.5 / 10.6
-//      ms on a rotation of 512^2 x 64, 7.6 / 7.7 ms at 384^2 x 48, 3.0 / 3.1 ms on
-//      a rotation of 256^2 x 32 (one row, in one wave of blocks: 15.4, 14.0, 5.4).
-//   4: thinner volumes, where rows in larger groups are carried along outside
-//      (256^2 x 16, 1440 views: 4.4 ms against 5.0 with 8; one row 6.3), and
-//      detectors of few rows.
-inline int forward_rows(const deam_geometry& g) {
-    if (g.n_rows < 2 || g.nx >= (1 << 21) || g.ny >= (1 << 21) || g.nz >= 2048) return 1;
-    double w = 0.0;  // largest row height in slices
-    for (int r : {0, g.n_rows - 1}) {
-        const double h = (r - (g.n_rows - 1) / 2.0 + g.row_offset) * g.row_pitch / g.dz;
-        w = h > w ? h : -h > w ? -h : w;
-    }
-    if (!(w < 2048.0)) return 1;
-    return g.n_rows > 4 && g.nz * g.dz >= 2.0 * g.n_rows * g.row_pitch * g.sid / g.sdd ? 8 : 4;
-}
+// Detector rows that a thread of the forward kernel projects at once: 1, 4 or 8.
+int forward_rows(const deam_geometry& g, int sms);
 // Blocks of four warps instead of eight: scans of one row per thread whose blocks of
 // eight are all resident at once, where whole blocks leave some SMs with a third more
 // work than others (128^2 x 360 views, 360 blocks of eight: 33 us, of four 29, of two

@@ -819,6 +819,44 @@ cudaError_t launch_layout(const float2* c, const float* m, int ones, float4* vol
     return cudaGetLastError();
 }
 
+// Rows in groups share a plane's terms and slices, at the price of fewer and longer
+// threads and of rows that are carried along outside the volume.  Times are of one
+// projection with 1 / 4 / 8 rows per thread, on 16 rows of 0.75 mm unless said.
+//   1: one row, or a volume or cone too large for the group's floor and step tests
+//      (indices below 2^21, heights below 2048 slices).
+//   1: rows that rise by more than 1.4 slices at the axis, so that they share no
+//      slices (256^2, 360 views: 1.88 slices 1.29 / 1.61 / 1.81 ms; 720 views: 1.36
+//      slices 1.82 / 1.78 / 2.03), and a volume below 0.6 of the height that the
+//      detector covers at the axis (256^2, 360 views: 2 slices 0.27 / 0.47 / 0.70 ms,
+//      8 slices 0.61 / 0.70 / 0.95, 12 slices 0.80 / 0.76 / 0.96).
+//   8: a volume at least twice as high as that: most rows meet it along the whole ray
+//      (a rotation of 512^2 x 64 8 rows 10.5 against 10.6 ms, 384^2 x 48 7.6 / 7.7,
+//      a rotation of 256^2 x 32 3.0 / 3.1), if its tiles fill the GPU.
+//   4: else, if these tiles fill it: 1.9 times over for rows that rise by a slice,
+//      fewer in proportion for rows that rise by less and share more (256^2 x 32, 300
+//      channels: 8 views 0.12 / 0.29 / 0.30 ms, 60 0.22 / 0.27 / 0.29, 180 0.45 / 0.46 /
+//      0.56, 360 0.79 / 0.68 / 0.75; with slices of 1.5 mm 60 views 0.21 / 0.20 / 0.24,
+//      180 0.44 / 0.39 / 0.43, 360 0.79 / 0.56 / 0.62).
+int forward_rows(const deam_geometry& g, int sms) {
+    if (g.n_rows < 2 || g.nx >= (1 << 21) || g.ny >= (1 << 21) || g.nz >= 2048) return 1;
+    double w = 0.0;  // largest row height in slices
+    for (int r : {0, g.n_rows - 1}) {
+        const double h = (r - (g.n_rows - 1) / 2.0 + g.row_offset) * g.row_pitch / g.dz;
+        w = h > w ? h : -h > w ? -h : w;
+    }
+    if (!(w < 2048.0)) return 1;
+    const double row = g.row_pitch * g.sid / g.sdd;  // height of a row at the axis
+    const double cover = g.n_rows * row, height = g.nz * g.dz;
+    if (row > 1.4 * g.dz || height < 0.6 * cover) return 1;
+    auto fills = [&](int rows) {
+        const double tiles = ((g.n_channels + 31) / 32) * (double)((g.n_rows + rows - 1) / rows) *
+                             ((g.n_views + kBlockViews - 1) / kBlockViews);
+        return tiles >= 1.9 * row / g.dz * fwd_min_blocks(rows) * sms;
+    };
+    if (g.n_rows > 4 && height >= 2.0 * cover && fills(8)) return 8;
+    return fills(4) ? 4 : 1;
+}
+
 bool forward_narrow(const Geo& G, int sms) {
     return G.fwd_rows == 1 && ray_tiles<1, kBlockViews, 1>(G) <= (long long)sms * fwd_min_blocks(1);
 }
