@@ -854,8 +854,11 @@ int deam_count_samples(deam_ctx* ctx, long long* n, void* stream) {
     DeviceGuard dg(ctx->device);
     cudaStream_t s = (cudaStream_t)stream;
     deam::FwdArgs A = fwd_args(ctx);
-    CK(deam::launch_forward(deam::FWD_COUNT, ctx->G, ctx->S, A, ctx->n_fwd_blocks, s));
-    CK(deam::launch_sum_partials(ctx->partial, ctx->n_fwd_blocks, ctx->scal + 1, 0, s));
+    // one wave that walks the tiles: the single block that adds up the partials takes
+    // longer than the count (256^2 x 2, 360 views x 16 x 512: 84 us with one per tile)
+    const int blocks = std::min(ctx->n_fwd_blocks, 152 * 4);
+    CK(deam::launch_forward(deam::FWD_COUNT, ctx->G, ctx->S, A, blocks, s));
+    CK(deam::launch_sum_partials(ctx->partial, blocks, ctx->scal + 1, 0, s));
     double v = 0.0;
     CK(cudaMemcpyAsync(&v, ctx->scal + 1, sizeof(double), cudaMemcpyDeviceToHost, s));
     CK(cudaStreamSynchronize(s));

@@ -1,4 +1,4 @@
-"""Scans of few rays: what a call costs follows what it works on."""
+"""Scans of few rays, thin volumes: what a call costs follows what it works on."""
 import dataclasses
 
 import pytest
@@ -49,3 +49,13 @@ def test_penalty_follows_the_voxels(pkg):
     assert _ms(lambda: few.penalty(c)) <= 1.5 * _ms(lambda: many.penalty(c))
     few.close()
     many.close()
+
+
+def test_count_follows_the_rays(pkg):
+    # the same rays through two slices and through 24: the count visits each ray once
+    # (a quarter is left for the clock's spread)
+    thin, thick = _scan(pkg, 360, 16, 500, nz=2), _scan(pkg, 360, 16, 500)
+    assert 0 < thin.count_samples() < thick.count_samples()
+    assert _ms(thin.count_samples, 25) <= 1.25 * _ms(thick.count_samples, 25)
+    thin.close()
+    thick.close()
