@@ -330,7 +330,8 @@ typedef struct deam_plan {
     int bwd_slab;   /* slices that a block of the backprojection takes (1: the kernel of single slices) */
     int bwd_groups; /* warps that share the views of a column */
     int bwd_rays;   /* rays of a view that one turn of the backprojection takes */
-    int reserved[4];
+    int bwd_views;  /* views that one turn takes */
+    int reserved[3];
 } deam_plan;
 
 /* The plan of the context (host memory). */

@@ -62,7 +62,7 @@ class deam_mar_params(C.Structure):
 
 class deam_plan(C.Structure):
     _fields_ = [("fwd_rows", C.c_int), ("bwd_slab", C.c_int), ("bwd_groups", C.c_int), ("bwd_rays", C.c_int),
-                ("reserved", C.c_int * 4)]
+                ("bwd_views", C.c_int), ("reserved", C.c_int * 3)]
 
 
 class DeamError(RuntimeError):

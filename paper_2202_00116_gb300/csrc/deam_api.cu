@@ -218,6 +218,28 @@ int2 deam::slab_view_range(const deam_geometry& g, int s, int slab, int ix0, int
     return make_int2((int)lo, (int)hi);
 }
 
+// How a context of geometry g backprojects (flat: all rays lie in the one slice).
+static deam::BwdPlan bwd_plan(const deam_geometry& g, bool flat, int sms) {
+    deam::BwdPlan p;
+    const long long patches = (long long)((g.nx + 7) / 8) * ((g.ny + 3) / 4);
+    if (g.nz == 1 && g.n_rows == 1) {
+        p.slab = 1;
+        p.flat = flat;
+        p.vs = patches >= 16LL * sms ? 8 : 16;
+        return p;
+    }
+    const int slab_class = deam::pick_slab(g.nz, g.n_rows, g.dz, g.row_pitch, g.sid, g.sdd);
+    p.slab = slab_class == 2 ? 2 : slab_class == 8 ? deam::kMidSlab : deam::kDeepSlab;
+    const int slabs = (g.nz + p.slab - 1) / p.slab;
+    const long long warps = patches * slabs, round = 20LL * sms;
+    p.vs = slab_class == 2 ? 4 : warps >= 8 * round ? 1 : warps >= 4 * round ? 2 : 4;
+    const int2 v = deam::slab_view_range(g, (slabs - 1) / 2, p.slab, 0, g.nx - 1, 0, g.ny - 1);
+    const int eights = (v.y - v.x + 8) / 8;
+    while (p.vs > 1 && eights < (warps * (p.vs / 2) >= round ? 2 * p.vs : p.vs / 2 + 1)) p.vs /= 2;
+    if (g.views_per_rotation < 16 || std::fabs(g.feed) >= 0.4 * g.dz * g.views_per_rotation) p.view_step = 1;
+    return p;
+}
+
 std::vector<int2> deam::tile_view_ranges(const deam_geometry& g, int slab, int tx, int ty) {
     const int ntx = (g.nx + tx - 1) / tx, nty = (g.ny + ty - 1) / ty, ns = (g.nz + slab - 1) / slab;
     std::vector<int2> v;
@@ -317,7 +339,7 @@ int deam_init(const deam_geometry* geom, const deam_spectra* spectra, const deam
     }
     // rays in the plane of the slice: no source height, no row height
     const bool flat = g.row_offset == 0.0 && std::all_of(vz.begin(), vz.end(), [](float z) { return z == 0.f; });
-    ctx->bwd = deam::bwd_plan(g, flat, sms);
+    ctx->bwd = bwd_plan(g, flat, sms);
     // per (slab, column tile) in the backprojector's block order
     // (a single slice is seen by all views)
     std::vector<int2> sv;
@@ -922,6 +944,7 @@ int deam_kernel_plan(const deam_ctx* ctx, deam_plan* plan) {
     plan->bwd_slab = ctx->bwd.slab;
     plan->bwd_groups = ctx->bwd.vs;
     plan->bwd_rays = ctx->bwd.slab > 1 ? deam::kRaysPerView : 1;
+    plan->bwd_views = ctx->bwd.slab > 1 ? ctx->bwd.view_step : ctx->bwd.vs == 8 ? 1 : 4;
     return DEAM_OK;
 }
 

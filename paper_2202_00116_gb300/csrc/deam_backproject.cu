@@ -155,7 +155,7 @@ struct Patch {
     float cx, cy;     // the corner that the lane looks from
     float u, ux, uy;  // of the lane's view: channel coordinate at the patch's centre, and its change over the patch
     float hw;         // half width of the window of the columns of any lane
-    int row0, row1;   // rows of a pair of views (2 w, 2 w + 1) that can reach the slab
+    int row0, row1;   // rows of the lane's view (STEP 2: of its pair 2 w, 2 w + 1) that can reach the slab
 
     __device__ __forceinline__ Patch(const Geo& G, int x0, int y0, int lane) {
         // lanes in 4 x 2 blocks of columns: the eight lanes of a 128-byte wavefront
@@ -173,6 +173,7 @@ struct Patch {
         cy = (float)(y0 + ((lane & 2) ? ey : 0));
     }
     // views vb .. vb + 7 (the last repeated beyond it): lane 4 w + c looks at view w
+    template <int STEP>
     __device__ __forceinline__ void look(const Geo& G, int vb, int last, int lane, float zlo, float zhi) {
         const CornerWindow win = corner_window<C>(G, min(vb + (lane >> 2), last), cx, cy, zlo, zhi);
         float lo = win.lo, hi = win.hi;
@@ -193,8 +194,10 @@ struct Patch {
         uy = 0.5f * ((c - a) + (d - b));
         hw += 0.25f * fabsf((b - a) - (d - c));
         if (C > 1) hw += 0.5f * (C - 1) * (fabsf(ux) * rx + fabsf(uy) * ry);
-        lo = fminf(lo, __shfl_xor_sync(0xffffffffu, lo, 4));  // both views of a pair
-        hi = fmaxf(hi, __shfl_xor_sync(0xffffffffu, hi, 4));
+        if (STEP > 1) {  // both views of a pair
+            lo = fminf(lo, __shfl_xor_sync(0xffffffffu, lo, 4));
+            hi = fmaxf(hi, __shfl_xor_sync(0xffffffffu, hi, 4));
+        }
         row0 = max(0, __float2int_ru(fminf(lo, (float)G.R)));
         row1 = min(G.R - 1, __float2int_rd(fmaxf(fminf(hi, (float)G.R), -1.f)));
     }
@@ -302,8 +305,8 @@ __device__ __forceinline__ bool finish_voxel(const Geo& G, const BwdArgs& A, lon
 
 // One (column tile, z-slab) of the gather backprojection: the work of one block
 // of VS groups of TX x TY threads.  Each group takes every VS-th eight views;
-// their sums are added in a fixed order (deterministic).
-template <int MODE, int SLAB, int TX, int TY, int VS>
+// their sums are added in a fixed order (deterministic).  A turn takes STEP views.
+template <int MODE, int SLAB, int TX, int TY, int VS, int STEP>
 __device__ __forceinline__ void bwd_tile(const Geo& G, const BwdArgs& A, Sums<MODE == BWD_UPDATE>* smem, int bx, int by,
                                          int slab) {
     // MODE: BWD_ADJOINT (A^T of two-component ray data), BWD_UPDATE (payload ->
@@ -329,20 +332,20 @@ __device__ __forceinline__ void bwd_tile(const Geo& G, const BwdArgs& A, Sums<MO
     const float fix = (float)ix, fiy = (float)iy;
     const float zlo = (float)(z0 - 1), zhi = (float)(z0 + SLAB);
     for (int vb = vrange.x + 8 * group; vb <= vrange.y; vb += 8 * VS) {
-        patch.look(G, vb, vrange.y, lane, zlo, zhi);
-        // Views in pairs: their samples of a row lie within a few hundredths of a
+        patch.template look<STEP>(G, vb, vrange.y, lane, zlo, zhi);
+        // Views in pairs (STEP 2): their samples of a row lie within a few hundredths of a
         // slice of each other, so nearly always all between the same two slices
         // (one read and write of their sums serves the rays of both)
         const int nv = min(8, vrange.y - vb + 1);
-        for (int w = 0; w < nv; w += 2) {
+        for (int w = 0; w < nv; w += STEP) {
             const int v = vb + w;
             const int r0 = __shfl_sync(0xffffffffu, patch.row0, 4 * w), r1 = __shfl_sync(0xffffffffu, patch.row1, 4 * w);
             int ka0, ka1, kb0, kb1;
             patch.channels(G, w, ka0, ka1);
-            patch.channels(G, w + 1, kb0, kb1);
+            patch.channels(G, w + STEP - 1, kb0, kb1);
             if (r0 > r1) continue;  // no row of these views reaches the slab
             if (!inside) continue;
-            const bool second = w + 1 < nv;
+            const bool second = STEP > 1 && w + 1 < nv;
             if (!second) kb1 = kb0 - 1;
             const float sza = __ldg(&G.view_z[v]), szb = __ldg(&G.view_z[second ? v + 1 : v]);
             const int n = max(ka1 - ka0, kb1 - kb0);
@@ -350,7 +353,7 @@ __device__ __forceinline__ void bwd_tile(const Geo& G, const BwdArgs& A, Sums<MO
                 Rays<G_> a, b;
                 float ta0 = INFINITY, ta1 = 0.f, tb0 = INFINITY, tb1 = 0.f;
                 load_rays<G_>(G, a, v, ka0 + j, ka1, fix, fiy, ta0, ta1);
-                load_rays<G_>(G, b, v + 1, kb0 + j, kb1, fix, fiy, tb0, tb1);
+                if (STEP > 1) load_rays<G_>(G, b, v + 1, kb0 + j, kb1, fix, fiy, tb0, tb1);
                 if (ta1 == 0.f && tb1 == 0.f) continue;
                 long long i = ((long long)v * G.R + r0) * G.K + j;
                 const long long next_view = (long long)G.R * G.K;
@@ -361,7 +364,7 @@ __device__ __forceinline__ void bwd_tile(const Geo& G, const BwdArgs& A, Sums<MO
 #pragma unroll 1
                 for (int r = r0; r <= r1; ++r) {
                     fetch_rays<MODE, G_>(G, A, a, i + ka0, P);
-                    fetch_rays<MODE, G_>(G, A, b, i + next_view + kb0, Q);
+                    if (STEP > 1) fetch_rays<MODE, G_>(G, A, b, i + next_view + kb0, Q);
                     const float om = __fmaf_rn(rf, G.domega, G.omega0);
                     const float rowf = MODE == BWD_ADJOINT ? __ldg(&G.row[r]).y : 1.f;
                     rf += 1.f;
@@ -386,7 +389,8 @@ __device__ __forceinline__ void bwd_tile(const Geo& G, const BwdArgs& A, Sums<MO
 #pragma unroll
                         for (int g = 0; g < G_; ++g) {
                             add_sample<FOUR>(lo, hi, row_fz(sza, om, a.t[g]) - f, a.c[g] * rowf, P[g]);
-                            add_sample<FOUR>(lo, hi, row_fz(szb, om, b.t[g]) - f, b.c[g] * rowf, Q[g]);
+                            if (STEP > 1)
+                                add_sample<FOUR>(lo, hi, row_fz(szb, om, b.t[g]) - f, b.c[g] * rowf, Q[g]);
                         }
                         acc[slot * NT] = lo;
                         acc[(slot + 1) * NT] = hi;
@@ -403,7 +407,8 @@ __device__ __forceinline__ void bwd_tile(const Geo& G, const BwdArgs& A, Sums<MO
                                 const float x = __fsub_rd(row_fz(sza, om, a.t[g]), fs);
                                 const float y = __fsub_rd(row_fz(szb, om, b.t[g]), fs);
                                 if (x >= 0.f && x < 1.f) add_sample<FOUR>(lo, hi, x, a.c[g] * rowf, P[g]);
-                                if (y >= 0.f && y < 1.f) add_sample<FOUR>(lo, hi, y, b.c[g] * rowf, Q[g]);
+                                if (STEP > 1 && y >= 0.f && y < 1.f)
+                                    add_sample<FOUR>(lo, hi, y, b.c[g] * rowf, Q[g]);
                             }
                             acc[s * NT] = lo;
                             acc[(s + 1) * NT] = hi;
@@ -448,7 +453,7 @@ __device__ __forceinline__ void slice_sums(const Geo& G, const BwdArgs& A, Patch
 #pragma unroll
     for (int j = 0; j < C * C; ++j) acc[j] = Sums<FOUR>{};
     for (int vb = 8 * group; vb < G.V; vb += 8 * VS) {
-        patch.look(G, vb, G.V - 1, lane, -1.f, 1.f);
+        patch.template look<2>(G, vb, G.V - 1, lane, -1.f, 1.f);
         const int nv = min(8, G.V - vb);
         for (int w = 0; w < nv; w += NV) {
             int k0[NV], k1[NV], n = -1;
@@ -582,7 +587,7 @@ struct BwdTile {
     static_assert(X * Y * VS == kBwdThreads, "view groups x columns fill the block");
 };
 
-template <int MODE, int SLAB, int VS>
+template <int MODE, int SLAB, int VS, int STEP>
 __global__ void __launch_bounds__(kBwdThreads, 5) bwd_kernel(const Geo G, const BwdArgs A) {
     constexpr int TX = BwdTile<VS>::X, TY = BwdTile<VS>::Y;
     __shared__ Sums<MODE == BWD_UPDATE> acc[(SLAB + 2) * kBwdThreads];
@@ -591,7 +596,7 @@ __global__ void __launch_bounds__(kBwdThreads, 5) bwd_kernel(const Geo G, const 
     const int bx = b % ntx;
     b /= ntx;
     const int by = b % nty;
-    bwd_tile<MODE, SLAB, TX, TY, VS>(G, A, acc, bx, by, b / nty);
+    bwd_tile<MODE, SLAB, TX, TY, VS, STEP>(G, A, acc, bx, by, b / nty);
 }
 
 // Batched scans: one launch takes the column tiles x slabs of every
@@ -611,27 +616,34 @@ __global__ void __launch_bounds__(TX* TY, 4) bwd_batch_kernel(const BatchDesc B)
         const int bx = (int)(lt % ntx);
         lt /= ntx;
         const int by = (int)(lt % nty);
-        bwd_tile<BWD_UPDATE, SLAB, TX, TY, 1>(G, A, acc, bx, by, (int)(lt / nty));
+        bwd_tile<BWD_UPDATE, SLAB, TX, TY, 1, 2>(G, A, acc, bx, by, (int)(lt / nty));
     }
 }
 
-template <int SLAB, int VS>
+template <int SLAB, int VS, int STEP>
 static cudaError_t launch_bwd(int mode, const Geo& G, const BwdArgs& A, cudaStream_t s) {
     constexpr int TX = BwdTile<VS>::X, TY = BwdTile<VS>::Y;
     const int blocks = ((G.nx + TX - 1) / TX) * ((G.ny + TY - 1) / TY) * ((G.nz + SLAB - 1) / SLAB);
-    if (mode == BWD_UPDATE) bwd_kernel<BWD_UPDATE, SLAB, VS><<<blocks, kBwdThreads, 0, s>>>(G, A);
-    else if (mode == BWD_GRADIENT) bwd_kernel<BWD_GRADIENT, SLAB, VS><<<blocks, kBwdThreads, 0, s>>>(G, A);
-    else bwd_kernel<BWD_ADJOINT, SLAB, VS><<<blocks, kBwdThreads, 0, s>>>(G, A);
+    if (mode == BWD_UPDATE) bwd_kernel<BWD_UPDATE, SLAB, VS, STEP><<<blocks, kBwdThreads, 0, s>>>(G, A);
+    else if (mode == BWD_GRADIENT) bwd_kernel<BWD_GRADIENT, SLAB, VS, STEP><<<blocks, kBwdThreads, 0, s>>>(G, A);
+    else bwd_kernel<BWD_ADJOINT, SLAB, VS, STEP><<<blocks, kBwdThreads, 0, s>>>(G, A);
     return cudaGetLastError();
+}
+
+template <int SLAB, int VS>
+static cudaError_t launch_slab(int mode, const BwdPlan& P, const Geo& G, const BwdArgs& A, cudaStream_t s) {
+    return P.view_step == 1 ? launch_bwd<SLAB, VS, 1>(mode, G, A, s) : launch_bwd<SLAB, VS, 2>(mode, G, A, s);
 }
 
 cudaError_t launch_backward(int mode, const BwdPlan& P, const Geo& G, const BwdArgs& A, cudaStream_t s) {
 #define DEAM_BWD(SL, VS) \
-    if (P.slab == SL && P.vs == VS) return launch_bwd<SL, VS>(mode, G, A, s);
+    if (P.slab == SL && P.vs == VS) return launch_slab<SL, VS>(mode, P, G, A, s);
     if (P.slab == 1) {
         if (P.flat) return P.vs == 8 ? launch_slice<2, 8, true>(mode, G, A, s) : launch_slice<1, 16, true>(mode, G, A, s);
         return P.vs == 8 ? launch_slice<2, 8, false>(mode, G, A, s) : launch_slice<1, 16, false>(mode, G, A, s);
     }
+    DEAM_BWD(2, 1)
+    DEAM_BWD(2, 2)
     DEAM_BWD(2, 4)
     DEAM_BWD(kMidSlab, 1)
     DEAM_BWD(kMidSlab, 2)

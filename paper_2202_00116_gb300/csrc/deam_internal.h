@@ -226,34 +226,27 @@ constexpr int kRaysPerView = 4;
 //   split so that the last, part-filled round weighs less: 4 warps against 1
 //   11.8 -> 9.9 ms (256^2 x 16: 2048 warps of columns), 11.7 -> 8.5 ms (256^2 x 32);
 //   2 against 1 19.4 -> 18.8 ms (384^2 x 48: 13,824); at 512^2 x 64 (32,768) 1 is
-//   as fast as 2 and 3 % faster than 4.
+//   as fast as 2 and 3 % faster than 4.  Warps that get no eight views of their own
+//   are idle, and where the columns alone fill the GPU each should have two eights, or
+//   setting up and adding the sums costs more than is gained: 256^2 x 32 with 1 / 2 / 4
+//   warps 8 views 92 / 122 / 206 us, 36 views 233 / 209 / 232, 90 views 469 / 417 / 430;
+//   96^2 x 8 (288 warps) 8 views 101 / 104 / 107, 24 views 194 / 149 / 105.
+//   view_step: two views a turn, but one where their samples lie in different slices:
+//   a source that moves by 0.4 slices or more from view to view (256^2 x 32, 0.1 / 0.3 /
+//   0.6 / 2 slices: two 1.48 / 0.63 / 0.36 / 0.26 ms, one 1.57 / 0.58 / 0.27 / 0.14),
+//   or fewer than 16 views per rotation (0.1 slices apart, 12 / 24 / 60 views: two 1.64 /
+//   1.51 / 1.48 ms, one 1.51 / 1.52 / 1.57).
 //   single slices (slab 1): with four 16 x 8 patches per SM, 2 x 2 columns per thread
 //   and 8 warps of views (4, 8, 16: 0.89, 0.85, 0.90 ms at 512^2); below, one column
 //   per thread and 16 (8: 55 us against 53 at 128^2).
 struct BwdPlan {
     int slab = 2, vs = 4;
+    int view_step = 2;  // views a turn of the row loop takes (slabs)
     bool flat = false;  // slab 1: all rays lie in the slice
 };
 constexpr int kMidSlab = 11, kDeepSlab = 16;
 constexpr int bwd_tile_x(int vs) { return vs == 1 ? 16 : 8; }
 constexpr int bwd_tile_y(int vs) { return vs == 4 ? 4 : 8; }
-inline BwdPlan bwd_plan(const deam_geometry& g, bool flat, int sms) {
-    BwdPlan p;
-    const long long patches = (long long)((g.nx + 7) / 8) * ((g.ny + 3) / 4);
-    if (g.nz == 1 && g.n_rows == 1) {
-        p.slab = 1;
-        p.flat = flat;
-        p.vs = patches >= 16LL * sms ? 8 : 16;
-        return p;
-    }
-    const int slab_class = pick_slab(g.nz, g.n_rows, g.dz, g.row_pitch, g.sid, g.sdd);
-    if (slab_class == 2) return p;
-    p.slab = slab_class == 8 ? kMidSlab : kDeepSlab;
-    const long long warps = patches * ((g.nz + p.slab - 1) / p.slab);
-    const long long round = 20LL * sms;
-    p.vs = warps >= 8 * round ? 1 : warps >= 4 * round ? 2 : 4;
-    return p;
-}
 long long forward_tiles(int shape, const Geo& G);
 long long backward_tiles(int shape, const Geo& G);
 cudaError_t launch_forward_batch(int shape, const BatchDesc& B, int grid, cudaStream_t s);
