@@ -237,6 +237,10 @@ static deam::BwdPlan bwd_plan(const deam_geometry& g, bool flat, int sms) {
     const int eights = (v.y - v.x + 8) / 8;
     while (p.vs > 1 && eights < (warps * (p.vs / 2) >= round ? 2 * p.vs : p.vs / 2 + 1)) p.vs /= 2;
     if (g.views_per_rotation < 16 || std::fabs(g.feed) >= 0.4 * g.dz * g.views_per_rotation) p.view_step = 1;
+    // rays of a view that pass within a voxel edge of a column at the axis (0.9: the
+    // mean cosine to their dominant axis)
+    const double taps = 0.9 * (g.dx + g.dy) / (g.sid * g.channel_pitch);
+    if (p.view_step == 2) p.rays = taps < 0.7 ? 1 : taps < 1.9 ? 2 : deam::kRaysPerView;
     return p;
 }
 
@@ -943,7 +947,7 @@ int deam_kernel_plan(const deam_ctx* ctx, deam_plan* plan) {
     plan->fwd_rows = ctx->G.fwd_rows;
     plan->bwd_slab = ctx->bwd.slab;
     plan->bwd_groups = ctx->bwd.vs;
-    plan->bwd_rays = ctx->bwd.slab > 1 ? deam::kRaysPerView : 1;
+    plan->bwd_rays = ctx->bwd.slab > 1 ? ctx->bwd.rays : 1;
     plan->bwd_views = ctx->bwd.slab > 1 ? ctx->bwd.view_step : ctx->bwd.vs == 8 ? 1 : 4;
     return DEAM_OK;
 }

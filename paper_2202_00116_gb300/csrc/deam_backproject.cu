@@ -305,8 +305,9 @@ __device__ __forceinline__ bool finish_voxel(const Geo& G, const BwdArgs& A, lon
 
 // One (column tile, z-slab) of the gather backprojection: the work of one block
 // of VS groups of TX x TY threads.  Each group takes every VS-th eight views;
-// their sums are added in a fixed order (deterministic).  A turn takes STEP views.
-template <int MODE, int SLAB, int TX, int TY, int VS, int STEP>
+// their sums are added in a fixed order (deterministic).  A turn takes RAYS rays of
+// STEP views.
+template <int MODE, int SLAB, int TX, int TY, int VS, int STEP, int RAYS>
 __device__ __forceinline__ void bwd_tile(const Geo& G, const BwdArgs& A, Sums<MODE == BWD_UPDATE>* smem, int bx, int by,
                                          int slab) {
     // MODE: BWD_ADJOINT (A^T of two-component ray data), BWD_UPDATE (payload ->
@@ -322,7 +323,7 @@ __device__ __forceinline__ void bwd_tile(const Geo& G, const BwdArgs& A, Sums<MO
     const int ix = patch.ix, iy = patch.iy;
     const bool inside = ix < G.nx && iy < G.ny;
     const int z0 = slab * SLAB;
-    constexpr int G_ = kRaysPerView;
+    constexpr int G_ = RAYS;
     Sums<FOUR>* acc = smem + group * (SLAB + 2) * NT + tid;  // slot s (slice z0 - 1 + s) at acc[s * NT]
 #pragma unroll
     for (int s = 0; s < SLAB + 2; ++s) acc[s * NT] = Sums<FOUR>{};
@@ -587,7 +588,7 @@ struct BwdTile {
     static_assert(X * Y * VS == kBwdThreads, "view groups x columns fill the block");
 };
 
-template <int MODE, int SLAB, int VS, int STEP>
+template <int MODE, int SLAB, int VS, int STEP, int RAYS>
 __global__ void __launch_bounds__(kBwdThreads, 5) bwd_kernel(const Geo G, const BwdArgs A) {
     constexpr int TX = BwdTile<VS>::X, TY = BwdTile<VS>::Y;
     __shared__ Sums<MODE == BWD_UPDATE> acc[(SLAB + 2) * kBwdThreads];
@@ -596,7 +597,7 @@ __global__ void __launch_bounds__(kBwdThreads, 5) bwd_kernel(const Geo G, const 
     const int bx = b % ntx;
     b /= ntx;
     const int by = b % nty;
-    bwd_tile<MODE, SLAB, TX, TY, VS, STEP>(G, A, acc, bx, by, b / nty);
+    bwd_tile<MODE, SLAB, TX, TY, VS, STEP, RAYS>(G, A, acc, bx, by, b / nty);
 }
 
 // Batched scans: one launch takes the column tiles x slabs of every
@@ -616,23 +617,26 @@ __global__ void __launch_bounds__(TX* TY, 4) bwd_batch_kernel(const BatchDesc B)
         const int bx = (int)(lt % ntx);
         lt /= ntx;
         const int by = (int)(lt % nty);
-        bwd_tile<BWD_UPDATE, SLAB, TX, TY, 1, 2>(G, A, acc, bx, by, (int)(lt / nty));
+        bwd_tile<BWD_UPDATE, SLAB, TX, TY, 1, 2, kRaysPerView>(G, A, acc, bx, by, (int)(lt / nty));
     }
 }
 
-template <int SLAB, int VS, int STEP>
+template <int SLAB, int VS, int STEP, int RAYS>
 static cudaError_t launch_bwd(int mode, const Geo& G, const BwdArgs& A, cudaStream_t s) {
     constexpr int TX = BwdTile<VS>::X, TY = BwdTile<VS>::Y;
     const int blocks = ((G.nx + TX - 1) / TX) * ((G.ny + TY - 1) / TY) * ((G.nz + SLAB - 1) / SLAB);
-    if (mode == BWD_UPDATE) bwd_kernel<BWD_UPDATE, SLAB, VS, STEP><<<blocks, kBwdThreads, 0, s>>>(G, A);
-    else if (mode == BWD_GRADIENT) bwd_kernel<BWD_GRADIENT, SLAB, VS, STEP><<<blocks, kBwdThreads, 0, s>>>(G, A);
-    else bwd_kernel<BWD_ADJOINT, SLAB, VS, STEP><<<blocks, kBwdThreads, 0, s>>>(G, A);
+    if (mode == BWD_UPDATE) bwd_kernel<BWD_UPDATE, SLAB, VS, STEP, RAYS><<<blocks, kBwdThreads, 0, s>>>(G, A);
+    else if (mode == BWD_GRADIENT) bwd_kernel<BWD_GRADIENT, SLAB, VS, STEP, RAYS><<<blocks, kBwdThreads, 0, s>>>(G, A);
+    else bwd_kernel<BWD_ADJOINT, SLAB, VS, STEP, RAYS><<<blocks, kBwdThreads, 0, s>>>(G, A);
     return cudaGetLastError();
 }
 
 template <int SLAB, int VS>
 static cudaError_t launch_slab(int mode, const BwdPlan& P, const Geo& G, const BwdArgs& A, cudaStream_t s) {
-    return P.view_step == 1 ? launch_bwd<SLAB, VS, 1>(mode, G, A, s) : launch_bwd<SLAB, VS, 2>(mode, G, A, s);
+    return P.view_step == 1 ? launch_bwd<SLAB, VS, 1, kRaysPerView>(mode, G, A, s)
+           : P.rays == 1    ? launch_bwd<SLAB, VS, 2, 1>(mode, G, A, s)
+           : P.rays == 2    ? launch_bwd<SLAB, VS, 2, 2>(mode, G, A, s)
+                            : launch_bwd<SLAB, VS, 2, kRaysPerView>(mode, G, A, s);
 }
 
 cudaError_t launch_backward(int mode, const BwdPlan& P, const Geo& G, const BwdArgs& A, cudaStream_t s) {

@@ -212,7 +212,13 @@ inline int pick_slab(int nz, int n_rows, double dz, double row_pitch, double sid
 }
 // Rays of a view that one turn of the row loop takes (more rays: more turns).
 // Four at 5 blocks of 128 threads per SM; three at 6 blocks are as fast at 2.6
-// rays per view and 8 % slower at 3.5 (384^2 x 48 on 816 channels).
+// rays per view and 8 % slower at 3.5 (384^2 x 48 on 816 channels).  Two where a
+// column is tapped by fewer than 1.9 rays of a view, one below 0.7 (bwd_plan), as a
+// turn costs its rays whether they tap or not: 360 views, 4 / 2 / 1 rays per turn at
+// 512^2 x 16 and 64 channels (0.2 rays) 3.18 / 2.30 / 2.08 ms, 200 (0.7) 3.54 / 2.50 /
+// 2.50, 300 (1.0) 3.60 / 2.59 / 3.28, 500 (1.7) 3.71 / 3.27; at 256^2 x 32 and 100
+// channels (0.7) 1.30 / 0.95 / 0.86, 200 (1.4) 1.37 / 1.02 / 1.45, 300 (2.1) 1.42 / 1.46,
+// 400 (2.7) 1.48 / 1.80.
 constexpr int kRaysPerView = 4;
 // How a single-scan context backprojects: z-slabs of `slab` slices, and the views
 // of a column shared out over `vs` warps (whose sums are added at the end).
@@ -242,6 +248,7 @@ constexpr int kRaysPerView = 4;
 struct BwdPlan {
     int slab = 2, vs = 4;
     int view_step = 2;  // views a turn of the row loop takes (slabs)
+    int rays = kRaysPerView;  // rays of each that it takes
     bool flat = false;  // slab 1: all rays lie in the slice
 };
 constexpr int kMidSlab = 11, kDeepSlab = 16;
