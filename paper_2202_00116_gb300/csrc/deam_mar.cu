@@ -9,6 +9,7 @@
 
 #include <algorithm>
 #include <string>
+#include <type_traits>
 #include <vector>
 
 #include "deam.h"
@@ -268,9 +269,11 @@ __global__ void __launch_bounds__(256) ramp_kernel(const float* p, long long nra
 // channel), compensated FP32 sums.  What a view and a column have in common (the
 // fan angle, its channel, the distance) is computed once for the slices whose
 // windows hold the view: 3.4 ms at 256^2 x 32 x 1160 views and two spectra with two
-// slices per thread, 4.3 ms with four (too few warps) and with one slice and scalar
-// loads of planar sinograms.
-template <int NS, int NZ>
+// slices per thread, 4.0 ms with one, 4.3 ms with four (too few warps) and with one
+// slice and scalar loads of planar sinograms.  Threads of one slice (small volumes,
+// single slices) need no look at the window, detectors of one row (ROWS false) no
+// height: 0.80 -> 0.67 ms at 512^2 x 720 views, 0.58 -> 0.39 at 64^2 x 16.
+template <int NS, int NZ, bool ROWS>
 __global__ void fbp_kernel(const float* __restrict__ q, const float4* __restrict__ vw, const float* __restrict__ vz,
                            const int2* __restrict__ win, const FbpGeo F, float* __restrict__ img) {
     typedef Lane<NS> L;
@@ -305,16 +308,16 @@ __global__ void fbp_kernel(const float* __restrict__ q, const float4* __restrict
         const int k0 = min((int)kf, F.K - 2);
         const float ak = kf - (float)k0;
         const T ak2 = L::dup(ak);
-        const float dist = sqrtf(L2);
+        const float dist = ROWS ? sqrtf(L2) : 0.f;
         const float inv = __frcp_rn(L2);
-        const float sz = __ldg(&vz[v]);
+        const float sz = ROWS ? __ldg(&vz[v]) : 0.f;
         const long long ev = (long long)v * F.R * F.K + k0;
 #pragma unroll
         for (int z = 0; z < NZ; ++z) {
-            if (v < w[z].x || v >= w[z].y) continue;
+            if (NZ > 1 && (v < w[z].x || v >= w[z].y)) continue;
             long long e = ev;
             T val;
-            if (F.R > 1) {
+            if (ROWS) {
                 const float wd = __fdiv_rn((Z[z] - sz) * F.sdd, dist);
                 const float rf = fminf(fmaxf(fmaf(wd, F.inv_rp, F.rc), 0.f), (float)(F.R - 1));
                 const int r0 = min((int)rf, F.R - 2);
@@ -426,10 +429,12 @@ cudaError_t filter(deam_ctx* ctx, const float* p, const float* chanw, const floa
     // 48 KB hold their rows, so that the threads with short windows take a second one
     // (two rows of 672 channels; one row, 0.3 to 0.7 ms slower of 15.5 for the whole
     // initialisation); a long row may need more, by opt-in (3072 channels of two
-    // spectra: 86 KB)
+    // spectra: 86 KB).  Few rows are spread over four blocks per SM first (360 rows of
+    // 256 channels: 16 us six to a block, 10 us one)
     const int fours = 2 * (((K + 1) / 2 + 3) / 4);
     const size_t room = 48 * 1024 > m.taps + m.row ? 48 * 1024 - m.taps : m.row;
-    const int per = (int)std::min<size_t>(std::max(1, 384 / fours), room / m.row);
+    const long long spread = std::max(1LL, nrows / (152 * 4));
+    const int per = (int)std::min<size_t>(std::min<long long>(std::max(1, 384 / fours), spread), room / m.row);
     const size_t sm = m.taps + per * m.row;
     if (sm > 48 * 1024) {
         // the limit is the kernel's, not this call's: always the longest row's, so that
@@ -527,10 +532,21 @@ int fbp(deam_ctx* ctx, const float* p, int n, float* q, float* img, cudaStream_t
     if (e == cudaSuccess)
         e = n == 2 ? filter<2>(ctx, p, d_chw, d_cone, d_ker, q, s) : filter<1>(ctx, p, d_chw, d_cone, d_ker, q, s);
     if (e == cudaSuccess) {
-        constexpr int NZ = 2;  // 1, 2, 4: 16.1, 15.4, 16.4 ms for the initialisation at 256^2 x 32
-        const dim3 grid((g.nx + 127) / 128, g.ny, (g.nz + NZ - 1) / NZ);
-        if (n == 2) fbp_kernel<2, NZ><<<grid, 128, 0, s>>>(q, d_vw, d_vz, d_win, F, img);
-        else fbp_kernel<1, NZ><<<grid, 128, 0, s>>>(q, d_vw, d_vz, d_win, F, img);
+        // two slices per thread where that leaves eight blocks per SM (128^2 x 24, 180
+        // views: 1536 blocks 0.16 ms against 0.17 with one; 96^2 x 16, 360 views: 768 blocks
+        // 0.29 against 0.21)
+        const long long pairs = (long long)((g.nx + 127) / 128) * g.ny * ((g.nz + 1) / 2);
+        auto run = [&](auto rows) {
+            const bool two = g.nz > 1 && pairs >= 152LL * 8;
+            const dim3 grid((g.nx + 127) / 128, g.ny, two ? (g.nz + 1) / 2 : g.nz);
+            constexpr bool ROWS = decltype(rows)::value;
+            if (n == 2 && two) fbp_kernel<2, 2, ROWS><<<grid, 128, 0, s>>>(q, d_vw, d_vz, d_win, F, img);
+            else if (n == 2) fbp_kernel<2, 1, ROWS><<<grid, 128, 0, s>>>(q, d_vw, d_vz, d_win, F, img);
+            else if (two) fbp_kernel<1, 2, ROWS><<<grid, 128, 0, s>>>(q, d_vw, d_vz, d_win, F, img);
+            else fbp_kernel<1, 1, ROWS><<<grid, 128, 0, s>>>(q, d_vw, d_vz, d_win, F, img);
+        };
+        if (R > 1) run(std::true_type{});
+        else run(std::false_type{});
         e = cudaGetLastError();
     }
     cudaError_t e2 = cudaFreeAsync(tab, s);
