@@ -532,12 +532,15 @@ int fbp(deam_ctx* ctx, const float* p, int n, float* q, float* img, cudaStream_t
     if (e == cudaSuccess)
         e = n == 2 ? filter<2>(ctx, p, d_chw, d_cone, d_ker, q, s) : filter<1>(ctx, p, d_chw, d_cone, d_ker, q, s);
     if (e == cudaSuccess) {
-        // two slices per thread where that leaves eight blocks per SM (128^2 x 24, 180
-        // views: 1536 blocks 0.16 ms against 0.17 with one; 96^2 x 16, 360 views: 768 blocks
-        // 0.29 against 0.21)
-        const long long pairs = (long long)((g.nx + 127) / 128) * g.ny * ((g.nz + 1) / 2);
+        // two slices per thread where that leaves 16 warps per SM with views to add
+        // (slices' windows, in rotations: 128^2 x 24 voxels, a rotation past 13 slices,
+        // 3277 warps 0.15 ms against 0.16 with one; 96^2 x 96, as far, 1843 warps 0.29 against
+        // 0.25; 128^2 x 8 1365 warps 0.28 against 0.20)
+        double seen = 0.0;
+        for (const int2& w : win) seen += w.y - w.x;
+        const double warps = (g.nx + 31) / 32 * (double)g.ny * seen / std::min(V, N) / 2.0;
         auto run = [&](auto rows) {
-            const bool two = g.nz > 1 && pairs >= 152LL * 8;
+            const bool two = g.nz > 1 && warps >= 152.0 * 16.0;
             const dim3 grid((g.nx + 127) / 128, g.ny, two ? (g.nz + 1) / 2 : g.nz);
             constexpr bool ROWS = decltype(rows)::value;
             if (n == 2 && two) fbp_kernel<2, 2, ROWS><<<grid, 128, 0, s>>>(q, d_vw, d_vz, d_win, F, img);

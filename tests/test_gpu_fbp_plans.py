@@ -1,4 +1,4 @@
-"""FBP with one and with two slices per thread (two from eight blocks per SM up), on
+"""FBP with one and with two slices per thread (two from 16 warps per SM up), on
 detectors of one row and of several, with odd and even slices; few rows spread over
 the GPU and many packed into blocks.  Against the FP64 oracle to the FBP's bar
 (relative L2 1e-4); the middle slice of a volume is the same bit for bit as that slice
@@ -37,7 +37,7 @@ def _scan(pkg, nx, nz, R, K, V):
 
 
 @pytest.mark.parametrize("R", [1, 4])
-@pytest.mark.parametrize("nx,nz", [(160, 3), (160, 9), (240, 11), (240, 12)])  # below and above 1216 pairs of slices
+@pytest.mark.parametrize("nx,nz", [(160, 3), (160, 9), (240, 11), (240, 12)])  # below and above 2432 warps
 def test_slices_per_thread(pkg, nx, nz, R):
     import oracle
     K, V = 200, 24
