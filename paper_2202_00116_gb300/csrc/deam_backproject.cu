@@ -588,8 +588,13 @@ struct BwdTile {
     static_assert(X * Y * VS == kBwdThreads, "view groups x columns fill the block");
 };
 
+// Blocks per SM: with one view a turn 80 registers do (16 views at 256^2 x 32, two
+// iterations 1.26 ms, 1.39 with five blocks; the c-step's FP64 logarithms weigh most
+// there and want the warps).
+constexpr int bwd_blocks(int step) { return step == 1 ? 6 : 5; }
+
 template <int MODE, int SLAB, int VS, int STEP, int RAYS>
-__global__ void __launch_bounds__(kBwdThreads, 5) bwd_kernel(const Geo G, const BwdArgs A) {
+__global__ void __launch_bounds__(kBwdThreads, bwd_blocks(STEP)) bwd_kernel(const Geo G, const BwdArgs A) {
     constexpr int TX = BwdTile<VS>::X, TY = BwdTile<VS>::Y;
     __shared__ Sums<MODE == BWD_UPDATE> acc[(SLAB + 2) * kBwdThreads];
     const int ntx = (G.nx + TX - 1) / TX, nty = (G.ny + TY - 1) / TY;
