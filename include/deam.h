@@ -106,7 +106,7 @@ typedef struct deam_options {
     int precision;          /* 0 (default): spectral sums in compensated FP32 and the objective in FP64;
                                1: plain FP32 sums and FP32 objective accumulation (for comparison).
                                Projection sampling is FP32 either way.  A batch holding a context
-                               with 1 runs its per-scan plan only (the persistent plan has only 0). */
+                               with 1 runs its per-scan plan only (the single-launch plan has only 0). */
     int reserved[6];        /* zero */
 } deam_options;
 
@@ -345,11 +345,12 @@ int deam_kernel_plan(const deam_ctx *ctx, deam_plan *plan);
  * One iteration of the batch is the MAR-DEAM iteration of deam_iterate for
  * every scan, run as one forward launch and one backprojection launch (per
  * slab class) over the work of all scans, captured once in a CUDA
- * graph and replayed.  autotune = 0 runs the persistent plan with default
- * shapes, 2 the per-scan plan (below) without tuning.  With autotune = 1 the first deam_batch_iterate times the
+ * graph and replayed (the single-launch plan).  autotune = 0 runs it with default
+ * shapes, 2 the per-scan plan (below) without tuning.  With autotune = 1 the first
+ * deam_batch_iterate times the
  * candidate ray-tile shapes (32 channels x rows x views) and backprojection
  * shapes (z-slab depth x column tile) on scratch copies of the images and keeps
- * the fastest, then times one iteration of that persistent plan against a plan
+ * the fastest, then times one iteration of that plan against one
  * that replays every scan's own kernels on parallel graph branches, and keeps
  * the faster plan; results equal deam_iterate's up to FP32 summation order. */
 typedef struct deam_batch deam_batch;
@@ -362,13 +363,13 @@ int deam_batch_create(deam_ctx *const *ctxs, int n, int autotune, deam_batch **o
  * The graph is re-captured when the image pointers change. */
 int deam_batch_iterate(deam_batch *b, float *const *c, int n_iter, double *hist, void *stream);
 
-/* Execution plan: *plan = 0 (persistent launches over all scans) or 1 (each
+/* Execution plan: *plan = 0 (one launch per stage over all scans) or 1 (each
  * scan's own kernels on a graph branch of its own), plan_ms[2] = the tuning
  * time of one captured iteration of each plan.  Chosen shapes of the
- * persistent plan: fwd_shape[2] = (rows, views) of the forward ray tile;
+ * single-launch plan: fwd_shape[2] = (rows, views) of the forward ray tile;
  * bwd_shapes[3][3] = (slab depth, tile x, tile y) for the slab classes 2, 8 and
  * 16 (a scan's class follows its geometry; zeros where no scan falls in a
- * class: each non-empty class gets its own persistent launch); fwd_ms[3],
+ * class: each non-empty class gets a launch of its own); fwd_ms[3],
  * bwd_ms[6] = the tuning times of every candidate (0 if not tuned).  Any
  * pointer may be NULL. */
 int deam_batch_info(deam_batch *b, int *plan, float *plan_ms, int *fwd_shape, int *bwd_shapes, float *fwd_ms,

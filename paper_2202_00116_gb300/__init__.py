@@ -504,12 +504,13 @@ def objective_noalloc(geo, I0, mu, c, d, mask, F, bowtie=None, mask_kind="bits")
 
 class DeamBatch:
     """Several scans (Deam contexts with data set) iterated together: one
-    persistent launch per stage over all scans, replayed from a CUDA graph,
+    launch per stage over all scans, replayed from a CUDA graph,
     tile shapes picked by timing on the first iterate (autotune=True)."""
 
     def __init__(self, scans, autotune=True, plan=None):
         """autotune=True: shapes and plan picked by timing on the first iterate;
-        False: the persistent plan with default shapes; plan="per_scan" forces
+        False: one launch per stage over all scans with default shapes (info()
+        calls this plan "persistent"); plan="per_scan" forces
         every scan's own kernels on graph branches (no tuning)."""
         import torch
         self.torch = torch

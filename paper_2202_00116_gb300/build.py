@@ -1,4 +1,4 @@
-"""Build libdeam.so in-tree with nvcc for sm_103a (no cmake, two translation
+"""Build libdeam.so in-tree with nvcc for sm_103a (no cmake, six translation
 units compiled in parallel, one -gencode)."""
 from __future__ import annotations
 

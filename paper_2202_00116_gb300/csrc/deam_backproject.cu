@@ -2,8 +2,9 @@
 // Sec. 2.3): b~_i(x) = sum_y h(x,y) B~_i(y) and delta_i(x) = sum_y h(x,y) D_i(y)
 // per voxel, fused with the log-ratio update c_i <- c_i - (1/Z) ln(b^_i / b~_i);
 // the gradient b^ - b~; and the plain transpose A^T y of two-component ray data.
-// h is Joseph's; the gather recomputes the forward kernel's samples exactly, so
-// the weights are the forward's transposed and no atomics are needed.
+// h is Joseph's; the gather recomputes the forward kernel's sample positions bit for
+// bit, so the weights are the forward's transposed (on single slices, and for heights
+// just below slice 0, to half a unit in the last place of 1) and no atomics are needed.
 #include <math.h>
 
 #include "deam_internal.h"
@@ -14,10 +15,11 @@ namespace deam {
 // Voxel-driven gather backprojection.  A thread owns one (ix, iy) column and the
 // SLAB slices of one z-slab, whose sums it keeps in shared memory ([slot][thread]:
 // conflict-free).  A warp owns an 8 x 4 patch of columns and takes the views that
-// can reach its slab two at a time: the channels whose rays tap a column come
-// from the fan angles of the patch's corners, and then a row of the detector is
-// one turn of the loop, which adds the samples of all the rays of both views
-// (2.6 rays per view and column at 512^2 x 816 channels).  These lie within a few
+// can reach its slab two at a time (STEP; one where they lie far apart): the channels
+// whose rays tap a column come from the fan angles of the patch's corners, and then a
+// row of the detector is one turn of the loop, which adds the samples of up to RAYS
+// rays of each view (2.6 rays per view and column at 512^2 x 816 channels; four, or
+// two and one on coarse fans).  These lie within a few
 // hundredths of a slice of each other, so nearly always all between the same two
 // slices, and one read and write of these two serves them all.  Sample positions
 // are the forward kernel's, bit for bit (same in-plane table, same explicitly
@@ -25,7 +27,9 @@ namespace deam {
 //
 // What bounds it: issue (0.6 per cycle and scheduler) and the latency of the
 // payload gathers with the 20 warps per SM that 96 registers allow, the L1 data
-// path being 60-70 % busy.  One ray at a time (two views abreast) cost twice the
+// path being 67-69 % busy.  The c-step's instances of four rays and two views spill
+// 56 bytes of stores and 128 of loads at 96 registers, the adjoint's 8 (ptxas);
+// 128 registers without spills at 4 blocks were as fast, 80 at 6 slower.  One ray at a time (two views abreast) cost twice the
 // shared-memory traffic, half the loads in flight and 70 instead of 31
 // instructions per (column, ray, row): 37.4 -> 23.3 ms on one rotation of the
 // 512^2 x 64 scan, 20.5 -> 8.5 ms on one of the 256^2 x 32 scan.  Measured and
@@ -546,7 +550,7 @@ __global__ void __launch_bounds__(32 * VS, 32 / VS) bwd_slice_kernel(const Geo G
             zero += 0.f * hi.x + 0.f * hi.y;
         }
     }
-    if (__any_sync(0xffffffffu, zero != 0.f)) 
+    if (__any_sync(0xffffffffu, zero != 0.f))
         slice_sums<MODE, C, VS, FLAT, true>(G, A, patch, inside, group, lane, acc);
     const float rowf = MODE == BWD_ADJOINT ? __ldg(&G.row[0]).y : 1.f;  // else the payload carries it
     unsigned long long skipped = 0;
