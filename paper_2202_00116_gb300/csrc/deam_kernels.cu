@@ -434,27 +434,42 @@ __device__ __forceinline__ bool near_trace(const Geo& G, const uint8_t* __restri
     return any != 0;
 }
 
-// The block that finishes last adds up the partial objectives, in a fixed order
-// whichever block it is, and clears what the iteration's next kernel counts in: the
-// launches for these two were 7 of the 105 us of an iteration at 128^2.  (Not with
-// rows in groups, whose launches take milliseconds: the code alone made them 3 %
-// slower.)
+// The block that finishes last adds up the partial objectives, whichever block it
+// is in the order of sum_partials_kernel and sum_ranges_kernel (256 strided sums, then
+// halves), so that a scan has the same objective to the bit alone and in a batch, and
+// clears what the iteration's next kernel counts in: the launches for these two were 7
+// of the 105 us of an iteration at 128^2.  (Not with rows in groups, whose launches
+// take milliseconds: the code alone made them 3 % slower.)
 template <int NT>
 __device__ __forceinline__ void last_block_total(const FwdArgs& A) {
+    static_assert(NT == 128 || NT == 256, "a thread takes one or two of the strided sums");
     __shared__ bool last;
-    if (threadIdx.x == 0) {
+    __shared__ double sh[256];
+    const int t = threadIdx.x;
+    if (t == 0) {
         __threadfence();  // the partial before the ticket
         last = atomicAdd(A.ticket, 1u) == gridDim.x - 1;
     }
     __syncthreads();
     if (!last) return;
     __threadfence();
-    double t = 0.0;
+    for (int j = t; j < 256; j += NT) {
+        double v = 0.0;
 #pragma unroll 8
-    for (int i = threadIdx.x; i < (int)gridDim.x; i += NT) t += __ldcg(&A.partial[i]);
-    t = block_reduce<NT, double>(t, false);
-    if (threadIdx.x == 0) {
-        *A.total = t;
+        for (int i = j; i < (int)gridDim.x; i += 256) v += __ldcg(&A.partial[i]);
+        sh[j] = v;
+    }
+    __syncthreads();
+    for (int h = 128; h >= 32; h >>= 1) {
+        if (t < h) sh[t] += sh[t + h];
+        __syncthreads();
+    }
+    if (t >= 32) return;
+    double v = sh[t];
+#pragma unroll
+    for (int h = 16; h > 0; h >>= 1) v += __shfl_down_sync(0xffffffffu, v, h);
+    if (t == 0) {
+        *A.total = v;
         *A.ticket = 0;
         if (A.clear) *A.clear = 0;
     }
