@@ -218,6 +218,14 @@ int2 deam::slab_view_range(const deam_geometry& g, int s, int slab, int ix0, int
     return make_int2((int)lo, (int)hi);
 }
 
+// Rays of a view that one turn of the backprojection's row loop takes, by those that
+// pass within a voxel edge of a column at the axis (0.9: the mean cosine to their
+// dominant axis).
+static int turn_rays(const deam_geometry& g) {
+    const double taps = 0.9 * (g.dx + g.dy) / (g.sid * g.channel_pitch);
+    return taps < 0.7 ? 1 : taps < 1.9 ? 2 : deam::kRaysPerView;
+}
+
 // How a context of geometry g backprojects (flat: all rays lie in the one slice).
 static deam::BwdPlan bwd_plan(const deam_geometry& g, bool flat, int sms) {
     deam::BwdPlan p;
@@ -237,10 +245,7 @@ static deam::BwdPlan bwd_plan(const deam_geometry& g, bool flat, int sms) {
     const int eights = (v.y - v.x + 8) / 8;
     while (p.vs > 1 && eights < (warps * (p.vs / 2) >= round ? 2 * p.vs : p.vs / 2 + 1)) p.vs /= 2;
     if (g.views_per_rotation < 16 || std::fabs(g.feed) >= 0.4 * g.dz * g.views_per_rotation) p.view_step = 1;
-    // rays of a view that pass within a voxel edge of a column at the axis (0.9: the
-    // mean cosine to their dominant axis)
-    const double taps = 0.9 * (g.dx + g.dy) / (g.sid * g.channel_pitch);
-    if (p.view_step == 2) p.rays = taps < 0.7 ? 1 : taps < 1.9 ? 2 : deam::kRaysPerView;
+    if (p.view_step == 2) p.rays = turn_rays(g);
     return p;
 }
 
@@ -361,6 +366,7 @@ int deam_init(const deam_geometry* geom, const deam_spectra* spectra, const deam
     G.inv_dgamma = (float)(1.0 / g.channel_pitch);
     G.fwd_rows = deam::forward_rows(g, sms);
     G.fwd_narrow = deam::forward_narrow(G, sms);
+    G.bwd_rays = turn_rays(g);
     ctx->n_fwd_blocks = deam::forward_blocks(G);
     G.vox_reach_mm = (float)(std::max(g.dx, g.dy) * 1.001);
     G.inv_sdd = (float)(1.0 / g.sdd);

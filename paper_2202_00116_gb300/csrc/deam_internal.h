@@ -22,6 +22,7 @@ struct Geo {
     int nx, ny, nz, V, R, K;
     int fwd_rows;            // rows a forward thread projects at once (forward_rows; host)
     int fwd_narrow;          // forward blocks of four warps (forward_narrow; host)
+    int bwd_rays;            // rays of a view that a turn of the batched backprojection takes (turn_rays)
     float dx, dy;            // voxel edge lengths (mm)
     float dx_sdd, dy_sdd;    // dx / sdd, dy / sdd
     float dx_dy, dy_dx;      // dx / dy, dy / dx
@@ -213,7 +214,7 @@ inline int pick_slab(int nz, int n_rows, double dz, double row_pitch, double sid
 // Rays of a view that one turn of the row loop takes (more rays: more turns).
 // Four at 5 blocks of 128 threads per SM; three at 6 blocks are as fast at 2.6
 // rays per view and 8 % slower at 3.5 (384^2 x 48 on 816 channels).  Two where a
-// column is tapped by fewer than 1.9 rays of a view, one below 0.7 (bwd_plan), as a
+// column is tapped by fewer than 1.9 rays of a view, one below 0.7 (turn_rays), as a
 // turn costs its rays whether they tap or not: 360 views, 4 / 2 / 1 rays per turn at
 // 512^2 x 16 and 64 channels (0.2 rays) 3.18 / 2.30 / 2.08 ms, 200 (0.7) 3.54 / 2.50 /
 // 2.50, 300 (1.0) 3.60 / 2.59 / 3.28, 500 (1.7) 3.71 / 3.27; at 256^2 x 32 and 100
