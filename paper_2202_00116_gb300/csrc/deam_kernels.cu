@@ -453,19 +453,20 @@ __device__ __forceinline__ void last_block_total(const FwdArgs& A) {
     __syncthreads();
     if (!last) return;
     __threadfence();
-    for (int j = t; j < 256; j += NT) {
-        double v = 0.0;
+    double v0 = 0.0, v1 = 0.0;  // sums t and (four warps) t + 128, their loads in flight together
 #pragma unroll 8
-        for (int i = j; i < (int)gridDim.x; i += 256) v += __ldcg(&A.partial[i]);
-        sh[j] = v;
+    for (int i = t; i < (int)gridDim.x; i += 256) {
+        v0 += __ldcg(&A.partial[i]);
+        if (NT == 128 && i + 128 < (int)gridDim.x) v1 += __ldcg(&A.partial[i + 128]);
     }
+    sh[t] = v0;
+    if (NT == 128) sh[t + 128] = v1;
     __syncthreads();
-    for (int h = 128; h >= 32; h >>= 1) {
-        if (t < h) sh[t] += sh[t + h];
-        __syncthreads();
-    }
     if (t >= 32) return;
-    double v = sh[t];
+    double q[4];
+#pragma unroll
+    for (int j = 0; j < 4; ++j) q[j] = sh[t + 32 * j] + sh[t + 32 * j + 128];
+    double v = (q[0] + q[2]) + (q[1] + q[3]);  // halves of 256, 128 and 64 without a barrier
 #pragma unroll
     for (int h = 16; h > 0; h >>= 1) v += __shfl_down_sync(0xffffffffu, v, h);
     if (t == 0) {
