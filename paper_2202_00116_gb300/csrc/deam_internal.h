@@ -226,9 +226,12 @@ constexpr int kRaysPerView = 4;
 //   slab: a deep slab costs less set-up per sample (a slab is visited by the views
 //   of slab + rows covered), a shallow one leaves more of the 256 KB to L1.  16
 //   against 13 slices, deep class: 18.7 / 19.8 ms at 384^2 x 48, 11.5 / 12.5 ms at
-//   256^2 x 16 x 1440 views, 22.9 / 23.1 ms on a rotation of 512^2 x 64.  11
-//   against 16 slices with several rows per slice: 8.5 / 9.8 ms on a rotation of
-//   256^2 x 32 x 672 channels.
+//   256^2 x 16 x 1440 views, 22.9 / 23.1 ms on a rotation of 512^2 x 64.  With
+//   rows of 2/3 of a slice or less 11 against 16: 8.5 / 9.8 ms on a rotation of
+//   256^2 x 32 x 672 channels; 11, 8 and 13 slices: there 8.6 / 9.3 / 9.0, 384^2 x 48
+//   12.0 / 12.4 / 11.3, 384^2 x 24 11.5 / 12.0 / 11.1, 512^2 x 64 10.6 / 11.2 / 10.6,
+//   192^2 x 40 2.76 / 2.79 / 2.61, 320^2 x 33 with one row 1.60 / 1.55 / 1.61 (the
+//   slices that the last slab leaves empty weigh as much as the depth).
 //   vs: 5 blocks of 4 warps run on an SM; below 8 rounds of the GPU the views are
 //   split so that the last, part-filled round weighs less: 4 warps against 1
 //   11.8 -> 9.9 ms (256^2 x 16: 2048 warps of columns), 11.7 -> 8.5 ms (256^2 x 32);
